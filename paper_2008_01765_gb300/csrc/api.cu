@@ -17,6 +17,7 @@ constexpr uint32_t kMaxK = 6;          // per-pass digit-count table is (2^k)^2 
 constexpr uint32_t kMaxPasses = 32;
 constexpr uint32_t kMaxLevels = 32;  // L < 32: slot indexes are 32-bit
 constexpr uint32_t kDefaultAttempts = 8;
+constexpr uint32_t kTicketLoads = 20;  // ctrl ticket of the final loads' prefix (0: LAST pass, 1..14: the sort)
 
 // Process-wide debug state. The trace buffer is read once per call under g_state_mu, so an
 // attach from one thread never tears a call's copy; the profiling events and totals are updated
@@ -143,6 +144,7 @@ struct Plan {
   uint32_t pass_i[kMaxPasses] = {};
   uint32_t pass_C[kMaxPasses] = {};
   bool pass_stream[kMaxPasses] = {};  // first / middle pass run by the streaming kernel (orp_stream.cu)
+  bool last_tile = false;             // LAST pass run by the packed-tile kernel (orp_last.cu)
   // workspace offsets
   size_t off_ctrl = 0, off_rec[2] = {0, 0}, off_tag[2] = {0, 0}, off_status = 0;
   size_t off_tmp = 0, off_hist = 0, off_dbase = 0, off_rstatus = 0, off_ord = 0, off_load = 0, total = 0;
@@ -184,7 +186,8 @@ uint32_t split_levels(uint32_t L, uint32_t kmid, uint32_t klast, uint32_t* pass_
   return 0;
 }
 
-bos_status make_plan(uint64_t n, const bos_params* p, bool sort, Plan* pl, uint32_t max_C = 16) {
+// tile: the last pass may be the packed-tile kernel (a shard's local levels have no last pass).
+bos_status make_plan(uint64_t n, const bos_params* p, bool sort, Plan* pl, uint32_t max_C = 16, bool tile = true) {
   if (!p) return BOS_ERR_INVALID;
   if (!((p->rec_bytes == 8 && p->key_bytes == 4) || (p->rec_bytes == 16 && p->key_bytes == 8)))
     return BOS_ERR_INVALID;
@@ -270,11 +273,6 @@ bos_status make_plan(uint64_t n, const bos_params* p, bool sort, Plan* pl, uint3
     static const double kMid[5] = {1.0, 1.371, 1.623, 1.919, 2.49};  // C = 1, 2, 4, 8, 16
     static const double kFirst[5] = {1.269, 1.496, 1.667, 2.168, 2.63};
     static const double kLast[5] = {1.219, 1.459, 1.723, 2.212, 2.63};
-    // Streaming kernel, k up to 8-9: set so that a streaming plan wins where it saves a pass. Its
-    // measured ratios at n = 2^30, Z = 1024 are 1.76 (first, k = 8) and 1.92 (paired middle), and
-    // with those the streaming plan still wins there; at small Z they would pick cluster plans
-    // that were never measured against it.
-    static const double kStreamFirst = 0.85, kStreamMid = 1.15;
     const uint32_t kcap = p->k ? p->k : kMaxKFast;
     auto c_for = [&](uint32_t k, bool last) -> uint32_t {  // smallest C holding k levels; 0: none
       if (k > kcap) return 0;
@@ -344,43 +342,33 @@ bos_status make_plan(uint64_t n, const bos_params* p, bool sort, Plan* pl, uint3
       }
       pl->pass_k[bnp - 1] = bl;
       pl->pass_C[bnp - 1] = c_for(bl, true);
-      // The streaming kernel (orp_stream.cu) takes the first and middle passes when that is
-      // cheaper: up to 8-9 levels a pass with no cluster, the last pass stays the cluster kernel
-      // (it needs its final buckets whole for the in-bin permutation). Costs in the same unit.
+      // The streaming kernels: orp_stream.cu takes the first and middle passes (5 to 8 levels each, no
+      // cluster), orp_last.cu or, beyond its tile, the cluster kernel the last one.
       const uint32_t kmin = orp_stream_min_k();
-      // An automatic plan keeps a batch to about 8 reals per output bucket on average (Z / 2^k in
-      // the first pass, Z / 2^(k+1) in a middle pass): more overrun the rings and the batch is
-      // redone in small rounds. A caller-given k is taken as given.
-      uint32_t lz = 0;
-      while ((1u << lz) < p->Z) ++lz;
-      const uint32_t kminf = p->k ? kmin : (lz >= 3 && lz - 3 > kmin ? lz - 3 : kmin);
-      const uint32_t kminm = p->k ? kmin : (lz >= 4 && lz - 4 > kmin ? lz - 4 : kmin);
       uint32_t ksf = (p->flags & BOS_FLAG_NO_STREAM) ? 0u : orp_stream_max_k(pl->R, p->Z, true, kMaxSmem);
       uint32_t ksm = ksf ? orp_stream_max_k(pl->R, p->Z, false, kMaxSmem) : 0u;
+      uint32_t kt = tile ? orp_last_max_k(pl->R, p->Z) : 0u;
       if (p->k) {  // a caller-given k caps every pass (k = 1 is the plain form)
         ksf = p->k >= kmin && ksf ? (ksf < p->k ? ksf : p->k) : 0u;
         ksm = p->k >= kmin && ksm ? (ksm < p->k ? ksm : p->k) : 0u;
+        kt = kt < p->k ? kt : p->k;
       }
-      if (ksf < kminf) ksf = 0;
-      if (ksm < kminm) ksm = 0;
-      double sbest = 1e30;
+      // the fewest passes; with the packed-tile last pass where it needs no more of them than the
+      // cluster one, and about the levels in the last pass that its kernel runs best
       uint32_t sl = 0, snp = 0;
-      for (uint32_t l = 1; ksf && l < L; ++l) {
-        const uint32_t Cl = c_for(l, true), S = L - l;
-        if (!Cl) continue;
-        for (uint32_t np = 1; np + 1 <= kMaxPasses; ++np) {
-          if (S < kminf + (np - 1) * kminm || (np > 1 && !ksm)) continue;
-          if (S > ksf + (np - 1) * ksm) continue;
-          const double c = kStreamFirst + (np - 1) * kStreamMid + kLast[ci(Cl)];
-          if (c < sbest - 1e-9) {
-            sbest = c;
-            sl = l;
-            snp = np;
-          }
-          break;  // more stream passes only cost more
-        }
+      const uint32_t kb = kt < orp_last_best_k(pl->R, p->Z) ? kt : orp_last_best_k(pl->R, p->Z);
+      for (uint32_t np = 1; ksf && !sl && np < bnp && (np == 1 || ksm); ++np) {
+        auto fits = [&](uint32_t l) { return l < L && L - l >= np * kmin && L - l <= ksf + (np - 1) * ksm; };
+        for (uint32_t l = kb; l > 0 && !sl; --l)
+          if (fits(l)) sl = l;
+        for (uint32_t l = kb + 1; l <= kt && !sl; ++l)
+          if (fits(l)) sl = l;
+        pl->last_tile = sl > 0;
+        for (uint32_t l = 1; l < L && !sl; ++l)
+          if (fits(l) && c_for(l, true)) sl = l;
+        snp = np;
       }
-      if (sl && sbest < bc - 1e-9) {
+      if (sl) {
         const uint32_t S = L - sl;
         pl->npass = snp + 1;
         // balanced split of S levels over snp passes, the first at most ksf, the others ksm
@@ -397,7 +385,7 @@ bos_status make_plan(uint64_t n, const bos_params* p, bool sort, Plan* pl, uint3
             }
         }
         pl->pass_k[snp] = sl;
-        pl->pass_C[snp] = c_for(sl, true);
+        pl->pass_C[snp] = pl->last_tile ? 1u : c_for(sl, true);
         pl->pass_stream[snp] = false;
       }
     }
@@ -475,6 +463,7 @@ bos_status device_plan(uint64_t n, const bos_params* p, bool sort, Plan* pl) {
     for (uint32_t x = 0; x < pl->npass && ok; ++x) {
       const int mode = (x == 0 ? kModeFirst : 0) | (x + 1 == pl->npass ? kModeLast : 0);
       if (pl->pass_stream[x]) continue;  // streaming passes: one CTA per SM, sized by the planner
+      if (pl->last_tile && x + 1 == pl->npass) continue;  // so is the packed-tile last pass
       ok = fast_occupancy_cached(pl->R, mode, pl->Z, pl->pass_k[x], pl->pass_C[x]) > 0;
     }
     if (ok) return BOS_OK;
@@ -692,6 +681,13 @@ bos_status run(const void* d_in, void* d_out, uint64_t n, const bos_params* p, v
         ta.buf_tag = a.buf_in_tag;
         ta.seed = p->seed;
         ta.trace = tr;
+        if (pl.last_tile) {
+          ta.status = a.status;
+          ta.ticket = &ctrl->tickets[kTicketLoads];
+          ta.ctrl = ctrl;
+          ta.skip_publish = a.skip_publish;
+          a.load = ta.load;
+        }
         const double tb = (double)pl.B * pl.Z * (2.0 + (first ? 0.0 : 4.0));  // rows out, tags in
         const int evt = prof_begin(st, kKPerm, tb);
         BOS_CUDA(launch_perm_table(ta, st, trace));
@@ -701,6 +697,8 @@ bos_status run(const void* d_in, void* d_out, uint64_t n, const bos_params* p, v
       const int ev = prof_begin(st, cls, in_b + out_b);
       if (pl.pass_stream[x])
         BOS_CUDA(launch_orp_stream(a, first, st, pl.R, trace));
+      else if (last && pl.last_tile)
+        BOS_CUDA(launch_orp_last(a, st, pl.R, trace));
       else if (pl.fast)
         BOS_CUDA(launch_orp_fast(a, mode, pl.pass_C[x], 0, st, pl.R, trace));
       else
@@ -1095,7 +1093,7 @@ bos_status shard_plan(uint64_t n, uint32_t G, const bos_params* p, ShardPlan* sp
   // the local levels: a plan over Bl buckets of L - g levels (n' fills them exactly)
   bos_params q = *p;
   q.flags &= ~(uint32_t)BOS_FLAG_PLAN_ONLY;
-  s = make_plan(sp->Bl * p->Z / 2, &q, false, &sp->lp);
+  s = make_plan(sp->Bl * p->Z / 2, &q, false, &sp->lp, 16, false);
   if (s != BOS_OK) return s;
   if (sp->lp.B != sp->Bl || sp->lp.L != full.L - g) return BOS_ERR_INVALID;
   // the final pass: g levels in one LAST pass

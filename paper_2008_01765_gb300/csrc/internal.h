@@ -32,6 +32,8 @@ struct PassArgs {
   const uint16_t* ord;      // LAST (persistent kernel): in-bin permutation table, B*Z slot indexes
   uint64_t bucket0;         // global index of local bucket 0 (a shard's buckets; 0 otherwise): the
                             // first pass's groups and the in-bin permutation keys use global indexes
+  const uint32_t* load;     // LAST (orp_last.cu): [B] reals per final bucket, counted ahead of the pass;
+                            // status[q] then holds the inclusive prefix of the subproblems' reals
 };
 
 // In-bin permutation table (perm_table.cu): row b < B lists final bucket b's slots in the order
@@ -48,6 +50,12 @@ struct PermTableArgs {
   uint32_t Z, attempt, i, k, L, buf_tag;
   uint64_t seed;
   Trace trace;
+  // prefix of the loads over the LAST subproblems (null: not wanted): status[q] = inclusive prefix of
+  // the reals of subproblems 0..q (decoupled look-back; zeroed words, a zeroed ticket)
+  unsigned long long* status;
+  uint32_t* ticket;
+  Ctrl* ctrl;
+  uint32_t skip_publish;  // debug: subproblem 0 never publishes
 };
 cudaError_t launch_perm_table(const PermTableArgs& a, cudaStream_t st, bool trace);
 
@@ -80,6 +88,12 @@ uint32_t orp_stream_smem_bytes(int R, uint32_t Z, uint32_t k, bool first);
 uint32_t orp_stream_max_k(int R, uint32_t Z, bool first, uint32_t smem_limit);
 inline uint32_t orp_stream_min_k() { return 5; }
 cudaError_t launch_orp_stream(const PassArgs& a, bool first, cudaStream_t st, int R, bool trace);
+
+// LAST pass with known final loads and table (orp_last.cu): a.load, a.status and a.ord filled by
+// launch_perm_table. Z a multiple of 32, <= 2048; k <= orp_last_max_k.
+uint32_t orp_last_max_k(int R, uint32_t Z);  // 0: the kernel cannot take this Z
+uint32_t orp_last_best_k(int R, uint32_t Z);  // the k a plan gives it when the pass count allows
+cudaError_t launch_orp_last(const PassArgs& a, cudaStream_t st, int R, bool trace);
 
 // The ORP with O(1) client storage (oblivious.cu, Section 4.1): bitonic-sort MergeSplits, one
 // launch per level, bitonic in-bin permutations, a scan of the loads and the strip.

@@ -45,18 +45,24 @@ constexpr int kLUnroll = 8;  // 16-byte tag loads in flight per thread
 
 // load[q*D + u] = reals of LAST subproblem q whose routing digit is u, for every subproblem q:
 // the reals of its input buckets s*2^i + t (s < D, q = G*2^i + t) with label bits [shift, shift+k)
-// equal to u, as the LAST pass counts them.
+// equal to u, as the LAST pass counts them. With a.status, the subproblems are taken by ticket and
+// status[q] gets the inclusive prefix of their reals (loads above Z, an overflow, count as Z).
 template <bool TRACE>
 __global__ void __launch_bounds__(kLT) final_load_kernel(PermTableArgs a) {
   extern __shared__ __align__(16) unsigned char smem[];
+  __shared__ uint32_t q_s;
   uint32_t* mcnt = reinterpret_cast<uint32_t*>(smem);
   const uint32_t Z = a.Z, D = 1u << a.k, cpb = Z / 4;  // 16-byte chunks per input bucket
   const uint32_t shift = a.L - a.i - a.k;
   const uint64_t units = a.B >> a.k;
   const int tid = threadIdx.x;
-  for (uint64_t q = blockIdx.x; q < units; q += gridDim.x) {
+  uint64_t q = blockIdx.x;
+  while (true) {
+    if (a.status && tid == 0) q_s = atomicAdd(a.ticket, 1u);
     for (uint32_t x = tid; x < D; x += kLT) mcnt[x] = 0;
     __syncthreads();
+    if (a.status) q = q_s;
+    if (q >= units) break;
     const uint64_t t = q & ((1ull << a.i) - 1), G = q >> a.i;
     if (TRACE && tid == 0)
       for (uint32_t s = 0; s < D; ++s)
@@ -84,7 +90,23 @@ __global__ void __launch_bounds__(kLT) final_load_kernel(PermTableArgs a) {
     }
     __syncthreads();
     for (uint32_t x = tid; x < D; x += kLT) a.load[q * D + x] = mcnt[x];
+    if (a.status && tid < 32) {
+      uint32_t total = 0;
+      for (uint32_t x = tid; x < D; x += 32) total += min(mcnt[x], Z);
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) total += __shfl_xor_sync(0xFFFFFFFFu, total, o);
+      if (tid == 0) {
+        if (q == 0) {
+          if (!a.skip_publish) st_status(a.status, st_word(kStIncl, 0, total));
+        } else {
+          st_status(a.status + q, st_word(kStAgg, 0, total));
+          const unsigned long long pre = lookback_window<8>(a.status, q, 1, 0, a.ctrl);
+          st_status(a.status + q, st_word(kStIncl, 0, pre + total));
+        }
+      }
+    }
     __syncthreads();  // mcnt is cleared for the next subproblem
+    q += gridDim.x;
   }
 }
 
