@@ -422,7 +422,7 @@ bos_status make_plan(uint64_t n, const bos_params* p, bool sort, Plan* pl, uint3
     pl->off_gstart = off;  off = align256(off + 65537 * 8);
     pl->off_rlist = off;   off = align256(off + 65537 * 4);
     pl->off_first = off;   off = align256(off + 257 * 8);
-    pl->off_meta = off;    off = align256(off + 32);
+    pl->off_meta = off;    off = align256(off + 64);
     pl->off_ridx = off;    off = align256(off + 2 * 65537 * 4);
     pl->off_spill = off;   off = align256(off + hybrid_spill_bytes(n, pl->R));
   }
@@ -713,7 +713,7 @@ bos_status run(const void* d_in, void* d_out, uint64_t n, const bos_params* p, v
         for (int stage = 2; stage <= 4; ++stage) {
           const int ev = prof_begin(st, stage == 4 ? kKLocal : kKMsd, 2.0 * n * pl.R, (uint32_t)stage);
           BOS_CUDA(launch_hybrid(ha, pl.R, stage, st));
-          if (stage == 4) count_launches(2);  // two warp-per-range launches and the CTA one
+          if (stage == 4) count_launches(6);  // one launch per range class and the fallback's
           prof_end(ev, st);
         }
       for (uint32_t d = 0; d < pl.digits; ++d) {  // skipped when the hybrid sort runs

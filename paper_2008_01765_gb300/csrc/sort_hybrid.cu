@@ -8,14 +8,14 @@
 //      when every value of the most significant varying digit dA holds at most kCap records;
 //      mode 3 when dA and dB (the next varying digit) are the key's top two digits and every
 //      (dA, dB) group holds at most kCap; otherwise mode 0, and the LSD passes run instead.
-//      Consecutive groups are packed into ranges of whole groups holding at most kCap records;
+//      Consecutive groups are packed into ranges of whole groups, listed by size class;
 //   3. modes 2, 3: a stable partition of the whole array by dA (the onesweep tile of the LSD pass);
 //   4. mode 3: a stable partition by dB inside every dA bucket (tiles per bucket, the look-back
 //      stopping at the bucket's first tile);
-//   5. every range is sorted on chip by (key, position) and its records gathered into place: a
-//      range of at most 1024 records by one warp in registers, a larger one by a CTA (a stable
-//      partition by the range's top varying digit in shared memory, then a warp sort of every
-//      sub-bucket; LSD passes over the varying digits when that does not fit).
+//   5. every range is sorted on chip by (key, position): a range of at most 256 records by one warp in
+//      registers, a larger one by a CTA sized for it (bin_sort_kernel: its records in shared memory,
+//      binned by key and ranked inside the bins); a range whose keys crowd a bin by
+//      local_sort_kernel (partition, warp sorts or LSD passes).
 // The partitions are stable and a range holds whole groups in key order, so sorting every range
 // by key sorts the array; ties keep the ORP's order. HBM passes: the mode's count (1 to 3) plus
 // the histogram, against 1 + the live digits for the LSD sort.
@@ -35,16 +35,29 @@ constexpr int kLWarps = kLThreads / 32;
 constexpr uint32_t kLocalMaxCtas = 192;  // spill buffers in the workspace (one per CTA)
 constexpr uint32_t kTagMsd1 = 12, kTagMsd2 = 13;
 constexpr uint32_t kTicketMsd1 = 10, kTicketMsd2 = 11, kTicketLocal = 12;
-constexpr uint32_t kWarpMax = 256;        // largest sub-bucket one warp sorts in registers
+constexpr uint32_t kWarpMax = 256;        // largest sub-bucket one warp sorts in registers (local_sort_kernel)
 constexpr int kSThreads = 256;            // warp-per-range kernel
-constexpr uint32_t kSmallMax = 1024;      // ranges of at most this many records: one warp each
-constexpr uint32_t kRangeList = 65537;    // the small ranges' list starts here in ridx
-constexpr uint32_t kTicketSmall = 13;     // and 14
-static_assert(kGroups <= 64u * kPlanThreads, "the plan keeps one bit per range in a 64-bit word");
+constexpr uint32_t kTicketClass = 13;     // .. 18: one per range class
+// Range classes by size, each with its own list and launch: 0 one warp per range (registers); 1..4 the
+// bin sort with the records in shared memory, 128 to 1024 threads (8, 4, 2 and 1 CTAs per SM); 5 the bin
+// sort with the keys in shared memory (1024 threads).
+constexpr uint32_t kClasses = 6, kMidClass = 3;
+constexpr uint32_t kFull = 20;            // a range with a fuller bin is sorted by LSD passes
+
+constexpr uint32_t kMetaLeft = 3, kMetaList = 4;  // meta words: ranges left over; list starts [kClasses + 1]
+template <int R, int CLS> struct Bin;
+template <int R> struct Bin<R, 0> { static constexpr uint32_t kMax = 256; };
+template <int R> struct Bin<R, 1> { static constexpr uint32_t kMax = 1056, kBits = 11; static constexpr int kT = 128, kCtas = 8; };
+template <int R> struct Bin<R, 2> { static constexpr uint32_t kMax = 2112, kBits = 12; static constexpr int kT = 256, kCtas = 4; };
+template <> struct Bin<16, 3> { static constexpr uint32_t kMax = 4352, kBits = 13; static constexpr int kT = 512, kCtas = 2; };
+template <> struct Bin<8, 3> { static constexpr uint32_t kMax = 6656, kBits = 13; static constexpr int kT = 512, kCtas = 2; };
+template <> struct Bin<16, 4> { static constexpr uint32_t kMax = 9216, kBits = 13; static constexpr int kT = 1024, kCtas = 1; };
+template <> struct Bin<8, 4> { static constexpr uint32_t kMax = 14848, kBits = 13; static constexpr int kT = 1024, kCtas = 1; };
 
 template <int R> struct Local;
 template <> struct Local<16> { static constexpr uint32_t kCap = 19456; };  // 10 B per record on chip
 template <> struct Local<8> { static constexpr uint32_t kCap = 28672; };   // 6 B per record on chip
+template <int R> struct Bin<R, 5> { static constexpr uint32_t kMax = Local<R>::kCap, kBits = 13; static constexpr int kT = 1024, kCtas = 1; };
 
 __host__ __device__ constexpr uint32_t al16(uint32_t x) { return (x + 15u) & ~15u; }
 
@@ -185,7 +198,6 @@ __global__ void __launch_bounds__(kPlanThreads) sort_plan_kernel(HybridArgs a) {
     a.meta[0] = mode;
     a.meta[1] = s_dA;
     a.meta[2] = s_dB;
-    a.meta[3] = 0;
   }
   __syncthreads();
   const uint32_t mode = s_mode, dA = s_dA;
@@ -199,64 +211,101 @@ __global__ void __launch_bounds__(kPlanThreads) sort_plan_kernel(HybridArgs a) {
   auto count = [&](uint32_t g) -> uint64_t {
     return mode == 1 ? a.n : mode == 2 ? (uint64_t)a.hist[dA * 256 + g] : (uint64_t)a.joint[g];
   };
-  // Ranges. Groups of more than kWarpMax records each get a range of their own (with the empty
-  // groups after it), so the on-chip sort splits them by the next digit into small sub-buckets.
-  // Smaller groups are packed: a range is a run of consecutive groups whose starts fall in one
-  // window of S records (at most S - 1 + gmax <= kCap records), broken at every top-digit value
-  // in mode 3, so that the groups are the on-chip sort's sub-buckets.
-  const bool single = gmax > kWarpMax;
-  const uint64_t S = (uint64_t)kCap - gmax + 1;
-  auto starts = [&](uint32_t g, uint64_t gs) -> bool {
+  // Ranges of whole groups. Groups that are large for a packed range get one each (with the empty
+  // groups after it); smaller ones are packed: a range is a run of consecutive groups whose starts
+  // fall in one window of S records (at most S - 1 + gmax <= P records). P gives every SM two ranges
+  // where n allows it, within the sizes of classes 1 to 3.
+  const uint32_t want = (uint32_t)(a.n / 304);
+  constexpr uint32_t kPmin = Bin<R, 1>::kMax, kPmax = Bin<R, kMidClass>::kMax;
+  const uint32_t P = want < kPmin ? kPmin : want < kPmax ? want : kPmax;
+  const bool single = gmax * 3 > P;
+  const uint32_t S = single ? 1u : P - (uint32_t)gmax + 1u;
+  auto starts = [&](uint32_t g, uint64_t gs) -> bool {  // gs < 2^31
     if (g == 0) return true;
     if (single) return count(g) > 0;
-    return (mode == 3 && (g & 255u) == 0) || gs / S != (gs - count(g - 1)) / S;
+    return (uint32_t)gs / S != (uint32_t)(gs - count(g - 1)) / S;
   };
-  const uint32_t per = (G + kPlanThreads - 1) / kPlanThreads;
-  const uint32_t g0 = tid * per < G ? tid * per : G, g1 = g0 + per < G ? g0 + per : G;
+  // Warp w takes the groups (later the ranges) [w per, (w + 1) per), 32 consecutive ones at a time: two
+  // passes over the groups (sums and range counts need the sums of the warps before), two over the
+  // ranges, every access coalesced. (One thread per 64 groups, as before: 0.37 ms in mode 3.)
+  const uint32_t lane = tid & 31u, warp = tid >> 5;
+  constexpr uint32_t kPW = kPlanThreads / 32;
+  const uint32_t per = ((G + kPW - 1) / kPW + 31u) & ~31u;
+  const uint32_t g0 = warp * per < G ? warp * per : G, g1 = g0 + per < G ? g0 + per : G;
   unsigned long long sum = 0, total = 0;
-  for (uint32_t g = g0; g < g1; ++g) sum += count(g);
-  const unsigned long long ex = plan_scan(sum, s_w, &total);
-  unsigned long long gs = ex;
+#pragma unroll 4
+  for (uint32_t g = g0 + lane; g < g1; g += 32) sum += count(g);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xFFFFFFFFu, sum, o);
+  const unsigned long long ex = __shfl_sync(0xFFFFFFFFu, plan_scan(lane == 0 ? sum : 0ull, s_w, &total), 0);
+  unsigned long long run = ex;
   uint32_t nr = 0;
-  for (uint32_t g = g0; g < g1; ++g) {
-    a.gstart[g] = gs;
-    nr += starts(g, gs) ? 1u : 0u;
-    gs += count(g);
-  }
+  auto walk = [&](auto&& each) {  // each(group, its start, is it a range's first group, lanes that are)
+    run = ex;
+    for (uint32_t b = g0; b < g1; b += 32) {
+      const uint32_t g = b + lane;
+      const uint32_t c = g < g1 ? (uint32_t)count(g) : 0u;
+      uint32_t incl = c;  // 32 groups of at most kCap records: 32 bits
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, incl, o);
+        if (lane >= (uint32_t)o) incl += y;
+      }
+      const unsigned long long gs = run + incl - c;
+      const bool st = g < g1 && starts(g, gs);
+      each(g, gs, st, __ballot_sync(0xFFFFFFFFu, st));
+      run += __shfl_sync(0xFFFFFFFFu, incl, 31);
+    }
+  };
+  walk([&](uint32_t g, unsigned long long gs, bool, uint32_t firsts) {
+    if (g < g1) a.gstart[g] = gs;
+    nr += __popc(firsts);
+  });
   if (tid == 0) a.gstart[G] = total;
   unsigned long long nranges = 0;
-  unsigned long long rx = plan_scan(nr, s_w, &nranges);
-  gs = ex;
-  for (uint32_t g = g0; g < g1; ++g) {
-    if (starts(g, gs)) a.rlist[rx++] = g;
-    gs += count(g);
-  }
-  if (tid == 0) {
-    a.rlist[nranges] = G;
-    a.meta[3] = (uint32_t)nranges;
-  }
+  uint32_t rx = (uint32_t)__shfl_sync(0xFFFFFFFFu, plan_scan(lane == 0 ? nr : 0ull, s_w, &nranges), 0);
+  walk([&](uint32_t g, unsigned long long, bool st, uint32_t firsts) {
+    if (st) a.rlist[rx + __popc(firsts & lanemask_lt())] = g;
+    rx += __popc(firsts);
+  });
+  if (tid == 0) a.rlist[nranges] = G;
   __syncthreads();  // the range list and the group starts are written
-  {  // ranges of at most kSmallMax records go to the warp kernel, larger ones to the CTA kernel
-    const uint32_t NR = (uint32_t)nranges, rper = (NR + kPlanThreads - 1) / kPlanThreads;
-    const uint32_t r0 = tid * rper < NR ? tid * rper : NR, r1 = r0 + rper < NR ? r0 + rper : NR;
-    // at most 64 ranges per thread (at most 65536 ranges): one bit each, set for a small range
-    unsigned long long small = 0;
-#pragma unroll 8
-    for (uint32_t r = r0; r < r1; ++r)
-      if (a.gstart[a.rlist[r + 1]] - a.gstart[a.rlist[r]] <= kSmallMax) small |= 1ull << (r - r0);
-    unsigned long long tsm = 0, tbg = 0;
-    const unsigned long long nsm = (unsigned long long)__popcll(small);
-    unsigned long long xs = plan_scan(nsm, s_w, &tsm);
-    unsigned long long xb = plan_scan((r1 - r0) - nsm, s_w, &tbg);
-    for (uint32_t r = r0; r < r1; ++r) {
-      if ((small >> (r - r0)) & 1ull)
-        a.ridx[kRangeList + xs++] = r;
-      else
-        a.ridx[xb++] = r;
+  {  // the ranges by class, one list after the other
+    const uint32_t NR = (uint32_t)nranges, rper = ((NR + kPW - 1) / kPW + 31u) & ~31u;
+    const uint32_t r0 = warp * rper < NR ? warp * rper : NR, r1 = r0 + rper < NR ? r0 + rper : NR;
+    auto cls = [&](uint32_t r) -> uint32_t {
+      const unsigned long long m = a.gstart[a.rlist[r + 1]] - a.gstart[a.rlist[r]];
+      return m <= Bin<R, 0>::kMax ? 0u : m <= Bin<R, 1>::kMax ? 1u : m <= Bin<R, 2>::kMax ? 2u
+             : m <= Bin<R, 3>::kMax ? 3u : m <= Bin<R, 4>::kMax ? 4u : 5u;
+    };
+    uint32_t nc[kClasses] = {0, 0, 0, 0, 0, 0}, at[kClasses], list = 0;
+#pragma unroll 4
+    for (uint32_t r = r0 + lane; r < r1; r += 32) {
+      const uint32_t c = cls(r);
+#pragma unroll
+      for (uint32_t y = 0; y < kClasses; ++y) nc[y] += c == y ? 1u : 0u;
+    }
+#pragma unroll
+    for (uint32_t y = 0; y < kClasses; ++y) {
+      unsigned long long tot = 0;
+      const uint32_t w = __reduce_add_sync(0xFFFFFFFFu, nc[y]);
+      at[y] = list + (uint32_t)__shfl_sync(0xFFFFFFFFu, plan_scan(lane == 0 ? w : 0ull, s_w, &tot), 0);
+      if (tid == 0) a.meta[kMetaList + y] = list;
+      list += (uint32_t)tot;
     }
     if (tid == 0) {
-      a.meta[4] = (uint32_t)tbg;
-      a.meta[5] = (uint32_t)tsm;
+      a.meta[kMetaList + kClasses] = list;
+      a.meta[kMetaLeft] = 0;  // ranges left to local_sort_kernel, listed in a.joint (dead after the plan)
+    }
+#pragma unroll 2
+    for (uint32_t b = r0; b < r1; b += 32) {
+      const uint32_t r = b + lane, c = r < r1 ? cls(r) : kClasses;
+#pragma unroll
+      for (uint32_t y = 0; y < kClasses; ++y) {
+        const uint32_t m = __ballot_sync(0xFFFFFFFFu, c == y);
+        if (c == y) a.ridx[at[y] + __popc(m & lanemask_lt())] = r;
+        at[y] += __popc(m);
+      }
     }
   }
   if (mode == 3) {  // MSD2 tiles: every dA bucket is cut into tiles of its own
@@ -449,7 +498,7 @@ __global__ void __launch_bounds__(kLThreads, 1) local_sort_kernel(HybridArgs a) 
   Rec* dst = sort_buf<R>(a, mode, mode);
   const uint32_t tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5;
   const uint32_t lt_mask = lanemask_lt();
-  const uint32_t nbig = a.meta[4];  // this kernel's ranges: those of more than kSmallMax records
+  const uint32_t nbig = a.meta[kMetaLeft];  // this kernel's ranges: those the bin sort left (a bin too full)
   // the digit read 1 counts: the top varying digit of a one-group range under this mode
   const uint32_t dspec = mode == 3 ? D - 3 : mode == 2 ? D - 2 : D - 1;
 
@@ -458,7 +507,7 @@ __global__ void __launch_bounds__(kLThreads, 1) local_sort_kernel(HybridArgs a) 
     __syncthreads();
     const uint32_t ti = misc[0];
     if (ti >= nbig) break;
-    const uint32_t r = a.ridx[ti];
+    const uint32_t r = a.joint[ti];
     const uint64_t lo = a.gstart[a.rlist[r]];
     const uint64_t m64 = a.gstart[a.rlist[r + 1]] - lo;
     if (m64 == 0 || m64 > kCap) {  // empty; or more than the plan allows (never: the counts bound it)
@@ -686,6 +735,345 @@ __global__ void __launch_bounds__(kLThreads, 1) local_sort_kernel(HybridArgs a) 
   }
 }
 
+// The ranges of classes 1..5: one CTA per range. The range is split by key, evenly between its smallest
+// and its largest one, into about as many bins as it has records: counts, a scan, and a scatter of (position, next
+// 32 key bits) into bin order by shared-memory atomics (any order inside a bin). Then every record
+// finds its rank among its bin's few members by (key, position), which is the stable order: 32 bits
+// decide almost every comparison, the whole keys the rest. Keys spread evenly over the bins give
+// at most about a dozen to a bin; a range with more than kFull in one (few distinct keys, clusters) is
+// ordered by LSD passes over the varying digits instead, positions moving between two arrays in
+// shared memory (class 5 has no room for them: such a range is left to local_sort_kernel).
+// n = 2^29 16-byte records (8192 per range): 6.43 ms, 14.9 ms for local_sort_kernel, which read a range
+// three times and sorted sub-buckets with bitonic networks; 40,000,001 records (packed ranges of about
+// 3600): 0.52 ms against 2.19 for one warp per group; n = 2^27 (2048 per range): 1.56 ms, 1.96 without
+// the class of 256 threads.
+// Bound by shared-memory wavefronts and the latency between a range's barriers.
+// Classes 1..4 hold the records in shared memory (one bulk copy in, gathered from there on the way
+// out; the CTA's next range is prefetched into L2 meanwhile), so each record is read and written once.
+// Class 5 holds the keys and gathers the records from a second read of the range.
+template <int R, int CLS>
+struct BinSmem {
+  using Key = typename RecT<R>::Key;
+  using B = Bin<R, CLS>;
+  static constexpr bool kRecs = CLS < 5;
+  static constexpr uint32_t kItem = kRecs ? (uint32_t)R : (uint32_t)sizeof(Key);
+  static constexpr uint32_t bins = al16(B::kMax * kItem + (kRecs && R == 8 ? 8 : 0));
+  static constexpr uint32_t rem = bins + (2u << B::kBits);
+  static constexpr uint32_t pl = rem + (kRecs ? al16(B::kMax * 4) : 0u);
+  static constexpr uint32_t wsum = pl + al16(B::kMax * 2);
+  static constexpr uint32_t total = wsum + 32 * 4 + 48;
+};
+
+template <int R, int CLS>
+__global__ void __launch_bounds__(Bin<R, CLS>::kT, Bin<R, CLS>::kCtas) bin_sort_kernel(HybridArgs a) {
+  using Rec = typename RecT<R>::T;
+  using Key = typename RecT<R>::Key;
+  using L = BinSmem<R, CLS>;
+  constexpr uint32_t T = Bin<R, CLS>::kT, kMax = Bin<R, CLS>::kMax, kBits = Bin<R, CLS>::kBits;
+  constexpr uint32_t kItems = (kMax + T - 1) / T;
+  constexpr uint32_t kU = 4;  // loads in flight per thread
+  constexpr bool kRecs = L::kRecs;
+  const uint32_t mode = a.ctrl->sort_mode;
+  if (mode == 0) return;
+  const uint32_t l0 = a.meta[kMetaList + CLS], nlist = a.meta[kMetaList + CLS + 1] - l0;
+  if (blockIdx.x >= nlist) return;
+  extern __shared__ __align__(16) unsigned char bsm[];
+  Rec* SR = reinterpret_cast<Rec*>(bsm);                          // [kMax] records (classes 1..4)
+  Key* SK = reinterpret_cast<Key*>(bsm);                          // [kMax] keys (class 5)
+  uint32_t* bins = reinterpret_cast<uint32_t*>(bsm + L::bins);    // [2^kBits / 2]: 16 bits each
+  uint32_t* rem = reinterpret_cast<uint32_t*>(bsm + L::rem);      // [kMax] next key bits in bin order (classes 1..4)
+  uint16_t* pl = reinterpret_cast<uint16_t*>(bsm + L::pl);        // [kMax] positions in bin order
+  uint32_t* wsum = reinterpret_cast<uint32_t*>(bsm + L::wsum);    // [32]
+  unsigned long long* red = reinterpret_cast<unsigned long long*>(wsum + 32);  // smallest and largest key
+  unsigned long long* bar = red + 2;
+  uint32_t* next = reinterpret_cast<uint32_t*>(red + 3);  // the CTA's next range
+  const Rec* src = sort_buf<R>(a, mode, mode - 1);
+  Rec* dst = sort_buf<R>(a, mode, mode);
+  const uint32_t tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5;
+  if (kRecs && tid == 0) {
+    mbar_init(smem_u32(bar), 1);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  uint32_t ti = blockIdx.x, parity = 0;  // the first range is the block's own, later ones come by ticket
+
+  while (true) {
+    const uint32_t r = a.ridx[l0 + ti];
+    const uint64_t lo = a.gstart[a.rlist[r]];
+    const uint64_t m64 = a.gstart[a.rlist[r + 1]] - lo;
+    const bool fits = m64 > 0 && m64 <= kMax;  // always: the plan lists only this class's sizes
+    const uint32_t m = fits ? (uint32_t)m64 : 0u;
+    const Rec* in = src + lo;
+    Rec* out = dst + lo;
+    // 8-byte records on an odd address start one slot into the array, so that the bulk copy's both
+    // ends are 16-byte aligned; the records at the odd ends are copied by threads
+    const uint32_t odd = kRecs && R == 8 ? (uint32_t)((reinterpret_cast<uintptr_t>(in) >> 3) & 1u) : 0u;
+    const uint32_t c0 = odd < m ? odd : m, c1 = R == 8 ? c0 + ((m - c0) & ~1u) : m;  // bulk part [c0, c1)
+    if (tid == 0) {
+      if (kRecs) {
+        mbar_expect_tx(smem_u32(bar), (c1 - c0) * R);
+        if (c1 > c0) tma_load(smem_u32(SR + odd + c0), in + c0, (c1 - c0) * R, smem_u32(bar));
+      }
+      if (!fits) atomicExch(&a.ctrl->bad, 1u);
+      red[0] = ~0ull;
+      red[1] = 0;
+      *next = gridDim.x + atomicAdd(&a.ctrl->tickets[kTicketClass + CLS], 1u);
+    }
+    const uint32_t lg = m > 1 ? 32u - (uint32_t)__clz(m - 1) : 0u, nb = lg < kBits ? (lg > 6 ? lg : 6u) : kBits;
+    for (uint32_t x = tid; x < (1u << nb) / 8; x += T) reinterpret_cast<uint4*>(bins)[x] = make_uint4(0, 0, 0, 0);
+    if (kRecs && R == 8) {
+      if (tid == 32 && c0 > 0) SR[odd] = in[0];
+      if (tid == 33 && c1 < m) SR[odd + c1] = in[c1];
+    }
+    __syncthreads();
+    const uint32_t tn = *next;
+    if (kRecs && tid == 0 && tn < nlist) {  // the next range on its way to L2
+      const uint32_t rn = a.ridx[l0 + tn];
+      const uint64_t ln = a.gstart[a.rlist[rn]], en = a.gstart[a.rlist[rn + 1]];
+      const uintptr_t p0 = reinterpret_cast<uintptr_t>(src + ln) & ~(uintptr_t)15;
+      const uint32_t nby = (uint32_t)((reinterpret_cast<uintptr_t>(src + en) - p0) & ~(uintptr_t)15);
+      if (nby) asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p0), "r"(nby) : "memory");
+    }
+    // ---- the smallest and the largest key ----
+    auto key_at = [&](uint32_t j) -> Key { return kRecs ? load_key<R>(SR + odd + j) : SK[j]; };
+    if (kRecs) mbar_wait(smem_u32(bar), parity, a.ctrl);
+    parity ^= 1u;
+    Key kmin = ~Key(0), kmax = Key(0);
+    for (uint32_t j0 = tid; j0 < m; j0 += kU * T) {
+      Key kk[kU];
+#pragma unroll
+      for (uint32_t u = 0; u < kU; ++u)
+        if (j0 + u * T < m) kk[u] = kRecs ? key_at(j0 + u * T) : load_key<R>(in + j0 + u * T);
+#pragma unroll
+      for (uint32_t u = 0; u < kU; ++u)
+        if (j0 + u * T < m) {
+          if (!kRecs) SK[j0 + u * T] = kk[u];
+          kmin = kk[u] < kmin ? kk[u] : kmin;
+          kmax = kk[u] > kmax ? kk[u] : kmax;
+        }
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      const Key x = __shfl_xor_sync(0xFFFFFFFFu, kmin, o), y = __shfl_xor_sync(0xFFFFFFFFu, kmax, o);
+      kmin = x < kmin ? x : kmin;
+      kmax = y > kmax ? y : kmax;
+    }
+    if (lane == 0) {
+      atomicMin(&red[0], (unsigned long long)kmin);
+      atomicMax(&red[1], (unsigned long long)kmax);
+    }
+    __syncthreads();
+    kmin = (Key)red[0];
+    kmax = (Key)red[1];
+    if (m < 2 || kmin == kmax) {  // every key equal: the range is already in order
+      for (uint32_t j = tid; j < m; j += T) out[j] = kRecs ? SR[odd + j] : in[j];
+    } else {
+      const uint32_t top = 64u - (uint32_t)__clzll((long long)(unsigned long long)(Key)(kmax - kmin));
+      const uint32_t sh = top > nb ? top - nb : 0u;
+      auto bin_of = [&](Key k) -> uint32_t { return (uint32_t)((Key)(k - kmin) >> sh); };
+      // the 32 bits below the bin's (all of them when sh <= 32)
+      auto rest_of = [&](Key k) -> uint32_t {
+        const unsigned long long d = (Key)(k - kmin);
+        return sh >= 32 ? (uint32_t)(d >> (sh - 32)) : sh ? (uint32_t)d << (32 - sh) : 0u;
+      };
+      // ---- counts, starts ----
+#pragma unroll 4
+      for (uint32_t j = tid; j < m; j += T) {
+        const uint32_t b = bin_of(key_at(j));
+        atomicAdd(&bins[b >> 1], 1u << ((b & 1u) * 16));
+      }
+      __syncthreads();
+      bool crowded;
+      {
+        constexpr uint32_t kPer = ((1u << kBits) / 2 + T - 1) / T;  // words per thread, consecutive
+        const uint32_t W = (1u << nb) / 2, w0 = tid * kPer;
+        uint32_t w[kPer], sum = 0, big = 0;
+        if constexpr (kPer % 4 == 0) {
+#pragma unroll
+          for (uint32_t x = 0; x < kPer; x += 4) {
+            const uint4 v = w0 + x < W ? reinterpret_cast<const uint4*>(bins)[(w0 + x) / 4] : make_uint4(0, 0, 0, 0);
+            w[x] = v.x, w[x + 1] = v.y, w[x + 2] = v.z, w[x + 3] = v.w;
+          }
+        } else {
+#pragma unroll
+          for (uint32_t x = 0; x < kPer; ++x) w[x] = w0 + x < W ? bins[w0 + x] : 0u;
+        }
+#pragma unroll
+        for (uint32_t x = 0; x < kPer; ++x) {
+          sum += (w[x] & 0xFFFFu) + (w[x] >> 16);
+          big |= ((w[x] & 0xFFFFu) > kFull || (w[x] >> 16) > kFull) ? 1u : 0u;
+        }
+        uint32_t incl = sum;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+          const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, incl, o);
+          if (lane >= (uint32_t)o) incl += y;
+        }
+        if (lane == 31) wsum[warp] = incl;
+        crowded = __syncthreads_or(big);
+        uint32_t run = __reduce_add_sync(0xFFFFFFFFu, lane < warp ? wsum[lane] : 0u) + incl - sum;
+#pragma unroll
+        for (uint32_t x = 0; x < kPer; ++x) {
+          const uint32_t c = w[x];
+          w[x] = run | (run + (c & 0xFFFFu)) << 16;
+          run += (c & 0xFFFFu) + (c >> 16);
+        }
+        if constexpr (kPer % 4 == 0) {
+#pragma unroll
+          for (uint32_t x = 0; x < kPer; x += 4)
+            if (w0 + x < W) reinterpret_cast<uint4*>(bins)[(w0 + x) / 4] = make_uint4(w[x], w[x + 1], w[x + 2], w[x + 3]);
+        } else {
+#pragma unroll
+          for (uint32_t x = 0; x < kPer; ++x)
+            if (w0 + x < W) bins[w0 + x] = w[x];
+        }
+      }
+      const uint16_t* order = pl;  // positions in key order
+      if (crowded && !kRecs) {  // the other kernel's range
+        if (tid == 0) a.joint[atomicAdd(&a.meta[kMetaLeft], 1u)] = r;
+        order = nullptr;
+      } else if (crowded) {
+        // ---- LSD passes. Warp w owns the positions [w c, (w + 1) c) of the current order; its counts
+        // of the 256 digit values, later its next places, are 16-bit words in the bins' memory ----
+        constexpr uint32_t W = T / 32;
+        uint16_t* cur = pl;
+        uint16_t* nxt = reinterpret_cast<uint16_t*>(rem);
+        const uint32_t c = ((m + W - 1) / W + 31u) & ~31u;
+        const uint32_t wlo = warp * c < m ? warp * c : m, whi = wlo + c < m ? wlo + c : m;
+        for (uint32_t j = tid; j < m; j += T) cur[j] = (uint16_t)j;
+        for (uint32_t d = 0; d * 8 < top; ++d) {
+          auto digit = [&](uint32_t j) -> uint32_t { return (uint32_t)((Key)(key_at(j) - kmin) >> (8 * d)) & 255u; };
+          __syncthreads();
+          for (uint32_t x = tid; x < W * 128; x += T) bins[x] = 0;
+          __syncthreads();
+          for (uint32_t q = wlo + lane; q < whi; q += 32) {
+            const uint32_t v = digit(cur[q]);
+            atomicAdd(&bins[warp * 128 + v / 2], 1u << ((v & 1u) * 16));
+          }
+          __syncthreads();
+          uint32_t tot = 0, incl = 0, same = 0;  // thread t < 128: the digit values 2t and 2t + 1, packed
+          if (tid < 128) {
+            for (uint32_t w = 0; w < W; ++w) tot += bins[w * 128 + tid];
+            same = (tot & 0xFFFFu) == m || (tot >> 16) == m ? 1u : 0u;
+            incl = (tot & 0xFFFFu) + (tot >> 16);
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+              const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, incl, o);
+              if (lane >= (uint32_t)o) incl += y;
+            }
+            if (lane == 31) wsum[warp] = incl;
+          }
+          if (__syncthreads_or(same)) continue;  // one value: the pass would change nothing
+          if (tid < 128) {
+            uint32_t run = incl - (tot & 0xFFFFu) - (tot >> 16);
+            for (uint32_t w = 0; w < warp; ++w) run += wsum[w];
+            run |= (run + (tot & 0xFFFFu)) << 16;
+            for (uint32_t w = 0; w < W; ++w) {
+              const uint32_t x = bins[w * 128 + tid];
+              bins[w * 128 + tid] = run;
+              run += x;
+            }
+          }
+          __syncthreads();
+          uint16_t* place = reinterpret_cast<uint16_t*>(bins) + warp * 256;
+          for (uint32_t b = wlo; b < whi; b += 32) {
+            const bool valid = b + lane < whi;
+            const uint32_t j = valid ? cur[b + lane] : 0u, v = valid ? digit(j) : 256u;
+            const uint32_t peers = row_peers(v, b + 32 <= whi);
+            const uint32_t lt = __popc(peers & lanemask_lt());
+            const uint32_t base = valid ? place[v] : 0u;
+            __syncwarp();
+            if (valid && lt == 0) place[v] = (uint16_t)(base + __popc(peers));
+            __syncwarp();
+            if (valid) nxt[base + lt] = (uint16_t)j;
+          }
+          uint16_t* t = cur;
+          cur = nxt;
+          nxt = t;
+        }
+        __syncthreads();
+        order = cur;
+      } else {
+        __syncthreads();
+        // ---- positions (and rests) into bin order; a bin's start becomes its end ----
+        uint32_t it[kItems];  // place in bin order << 16 | bin
+#pragma unroll
+        for (uint32_t i = 0; i < kItems; ++i) {
+          const uint32_t j = tid + i * T;
+          if (j < m) {
+            const Key k = key_at(j);
+            const uint32_t b = bin_of(k), hs = (b & 1u) * 16;
+            const uint32_t p = (atomicAdd(&bins[b >> 1], 1u << hs) >> hs) & 0xFFFFu;
+            pl[p] = (uint16_t)j;
+            if (kRecs) rem[p] = rest_of(k);
+            it[i] = p << 16 | b;
+          }
+        }
+        __syncthreads();
+        // ---- every record's rank in its bin ----
+#pragma unroll
+        for (uint32_t i = 0; i < kItems; ++i) {
+          const uint32_t j = tid + i * T;
+          if (j < m) {
+            const uint32_t b = it[i] & 0xFFFFu, p = it[i] >> 16;
+            const uint32_t e = (bins[b >> 1] >> ((b & 1u) * 16)) & 0xFFFFu;
+            const uint32_t s = b ? (bins[(b - 1) >> 1] >> (((b - 1) & 1u) * 16)) & 0xFFFFu : 0u;
+            uint32_t rank = s;
+            if (kRecs) {
+              const uint32_t mine = rem[p];
+              for (uint32_t q = s; q < e; ++q) {
+                const uint32_t x = rem[q];
+                rank += x < mine ? 1u : 0u;
+                if (x == mine && q != p) {  // equal so far: the whole keys, then the positions
+                  const uint32_t j2 = pl[q];
+                  const Key k = key_at(j), k2 = key_at(j2);
+                  rank += (k2 < k || (k2 == k && j2 < j)) ? 1u : 0u;
+                }
+              }
+            } else {
+              const Key k = key_at(j);
+              for (uint32_t q = s; q < e; ++q) {
+                const uint32_t j2 = pl[q];
+                const Key k2 = key_at(j2);
+                rank += (k2 < k || (k2 == k && j2 < j)) ? 1u : 0u;
+              }
+            }
+            it[i] = rank;
+          }
+        }
+        __syncthreads();
+#pragma unroll
+        for (uint32_t i = 0; i < kItems; ++i)
+          if (tid + i * T < m) pl[it[i]] = (uint16_t)(tid + i * T);
+        __syncthreads();
+      }
+      if (order) {  // ---- the records in key order ----
+        for (uint32_t j0 = tid; j0 < m; j0 += kU * T) {
+          Rec v[kU];
+#pragma unroll
+          for (uint32_t u = 0; u < kU; ++u)
+            if (j0 + u * T < m) v[u] = kRecs ? SR[odd + order[j0 + u * T]] : in[order[j0 + u * T]];
+#pragma unroll
+          for (uint32_t u = 0; u < kU; ++u)
+            if (j0 + u * T < m) out[j0 + u * T] = v[u];
+        }
+      }
+    }
+    ti = tn;
+    if (ti >= nlist) break;
+    __syncthreads();  // the arrays are free
+  }
+}
+
+template <int R, int CLS>
+cudaError_t launch_bins(const HybridArgs& a, int sms, cudaStream_t st) {
+  auto kern = bin_sort_kernel<R, CLS>;
+  static_assert(Bin<R, CLS>::kCtas * (BinSmem<R, CLS>::total + 1024) <= 233472, "the CTAs of this class fit an SM");
+  const cudaError_t e = set_smem_optin(kern);
+  if (e != cudaSuccess) return e;
+  kern<<<(unsigned)(sms * Bin<R, CLS>::kCtas), Bin<R, CLS>::kT, BinSmem<R, CLS>::total, st>>>(a);
+  return cudaGetLastError();
+}
+
 // Ascending bitonic sort of (key, position) pairs in registers, the same network as warp_sort:
 // lane l holds elements l * EPL .. l * EPL + EPL - 1. Positions are distinct; padding is the
 // largest pair. The stage loops stay rolled (one body per partner distance below EPL and one for
@@ -739,9 +1127,7 @@ __device__ __forceinline__ void warp_sort_pairs(Key (&k)[EPL], uint32_t (&x)[EPL
       if (j >= (uint32_t)EPL) pair_stage_cross<Key, EPL>(k, x, lane, kk, j / EPL);
       else if (j == 1) pair_stage_lane<Key, EPL, 1>(k, x, lane, kk);
       else if (j == 2) pair_stage_lane<Key, EPL, 2>(k, x, lane, kk);
-      else if (j == 4) pair_stage_lane<Key, EPL, 4>(k, x, lane, kk);
-      else if (j == 8) pair_stage_lane<Key, EPL, 8>(k, x, lane, kk);
-      else pair_stage_lane<Key, EPL, 16>(k, x, lane, kk);
+      else pair_stage_lane<Key, EPL, 4>(k, x, lane, kk);
     }
   }
 }
@@ -772,44 +1158,36 @@ __device__ __forceinline__ void small_range(const typename RecT<R>::T* in, typen
   __syncwarp();
 }
 
-// The ranges of at most kSmallMax records (many small groups: n between about 2^22 and 2^28 for
-// 16-byte records), a warp each, taken by ticket; no block-wide barrier. Two launches share the
-// list: BIG = false sorts the ranges of at most 512 records (16 pairs per lane at most, so more
-// warps fit an SM), BIG = true those of 513 to 1024 (32 pairs per lane).
-template <int R, bool BIG>
+// The ranges of class 0 (many small groups), a warp each, taken by ticket; no block-wide barrier.
+template <int R>
 __global__ void __launch_bounds__(kSThreads) local_small_kernel(HybridArgs a) {
   using Rec = typename RecT<R>::T;
-  constexpr uint32_t kMax = BIG ? 1024u : 512u;
+  constexpr uint32_t kMax = Bin<R, 0>::kMax;
   const uint32_t mode = a.ctrl->sort_mode;
   if (mode == 0) return;
   __shared__ uint16_t sidx[kSThreads / 32][kMax];
   const Rec* src = sort_buf<R>(a, mode, mode - 1);
   Rec* dst = sort_buf<R>(a, mode, mode);
   const uint32_t lane = threadIdx.x & 31u, w = threadIdx.x >> 5;
-  const uint32_t nsmall = a.meta[5];
+  const uint32_t l0 = a.meta[kMetaList], nlist = a.meta[kMetaList + 1] - l0;
   while (true) {
     uint32_t t = 0;
-    if (lane == 0) t = atomicAdd(&a.ctrl->tickets[BIG ? kTicketSmall + 1 : kTicketSmall], 1u);
+    if (lane == 0) t = atomicAdd(&a.ctrl->tickets[kTicketClass], 1u);
     t = __shfl_sync(0xFFFFFFFFu, t, 0);
-    if (t >= nsmall) break;
-    const uint32_t r = a.ridx[kRangeList + t];
+    if (t >= nlist) break;
+    const uint32_t r = a.ridx[l0 + t];
     const uint64_t lo = a.gstart[a.rlist[r]];
     const uint64_t m64 = a.gstart[a.rlist[r + 1]] - lo;
-    if (m64 > kSmallMax) {  // never: the plan lists only small ranges here
+    if (m64 > kMax) {  // never: the plan lists only small ranges here
       if (lane == 0) atomicExch(&a.ctrl->bad, 1u);
       continue;
     }
     const uint32_t m = (uint32_t)m64;
-    if (m == 0 || (m > 512) != BIG) continue;  // the other launch's range
-    if constexpr (BIG) {
-      small_range<R, 32>(src + lo, dst + lo, m, sidx[w], lane);
-    } else {
-      if (m <= 32) small_range<R, 1>(src + lo, dst + lo, m, sidx[w], lane);
-      else if (m <= 64) small_range<R, 2>(src + lo, dst + lo, m, sidx[w], lane);
-      else if (m <= 128) small_range<R, 4>(src + lo, dst + lo, m, sidx[w], lane);
-      else if (m <= 256) small_range<R, 8>(src + lo, dst + lo, m, sidx[w], lane);
-      else small_range<R, 16>(src + lo, dst + lo, m, sidx[w], lane);
-    }
+    if (m == 0) continue;
+    if (m <= 32) small_range<R, 1>(src + lo, dst + lo, m, sidx[w], lane);
+    else if (m <= 64) small_range<R, 2>(src + lo, dst + lo, m, sidx[w], lane);
+    else if (m <= 128) small_range<R, 4>(src + lo, dst + lo, m, sidx[w], lane);
+    else small_range<R, 8>(src + lo, dst + lo, m, sidx[w], lane);
   }
 }
 
@@ -855,10 +1233,13 @@ cudaError_t launch_r(const HybridArgs& a, int stage, cudaStream_t st) {
       break;
     }
     default: {
-      local_small_kernel<R, false><<<(unsigned)sms * 8, kSThreads, 0, st>>>(a);
+      local_small_kernel<R><<<(unsigned)sms * 8, kSThreads, 0, st>>>(a);
       if ((e = cudaGetLastError()) != cudaSuccess) return e;
-      local_small_kernel<R, true><<<(unsigned)sms * 4, kSThreads, 0, st>>>(a);
-      if ((e = cudaGetLastError()) != cudaSuccess) return e;
+      if ((e = launch_bins<R, 1>(a, sms, st)) != cudaSuccess) return e;
+      if ((e = launch_bins<R, 2>(a, sms, st)) != cudaSuccess) return e;
+      if ((e = launch_bins<R, 3>(a, sms, st)) != cudaSuccess) return e;
+      if ((e = launch_bins<R, 4>(a, sms, st)) != cudaSuccess) return e;
+      if ((e = launch_bins<R, 5>(a, sms, st)) != cudaSuccess) return e;
       const uint32_t smem = local_smem_bytes<R>();
       if ((e = cudaFuncSetAttribute(local_sort_kernel<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) !=
           cudaSuccess)
