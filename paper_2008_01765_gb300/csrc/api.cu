@@ -17,6 +17,8 @@ constexpr uint32_t kMaxK = 6;          // per-pass digit-count table is (2^k)^2 
 constexpr uint32_t kMaxPasses = 32;
 constexpr uint32_t kMaxLevels = 32;  // L < 32: slot indexes are 32-bit
 constexpr uint32_t kDefaultAttempts = 8;
+constexpr uint32_t kMaxStreamK = 8;     // most levels of a streaming pass
+constexpr uint32_t kPlanSms = 152;     // SMs the planner counts on
 constexpr uint32_t kTicketLoads = 20;  // ctrl ticket of the final loads' prefix (0: LAST pass, 1..14: the sort)
 
 // Process-wide debug state. The trace buffer is read once per call under g_state_mu, so an
@@ -99,6 +101,102 @@ cudaError_t zero_async(void* p, size_t bytes, cudaStream_t st) {
   zero_kernel<<<grid, 256, 0, st>>>(static_cast<unsigned char*>(p), bytes);
   return cudaGetLastError();
 }
+
+// Zeroes up to six segments with one launch (each 16-byte aligned, its size rounded up to 16 bytes: the
+// workspace's regions are padded to 256).
+struct ZeroSegs {
+  uint4* p[6];
+  size_t words[6];
+};
+__global__ void zero_segs_kernel(ZeroSegs z) {
+  for (int s = 0; s < 6; ++s)
+    for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < z.words[s]; i += (size_t)gridDim.x * blockDim.x)
+      z.p[s][i] = make_uint4(0, 0, 0, 0);
+}
+struct Zeroer {
+  ZeroSegs z{};
+  int n = 0;
+  size_t words = 0;
+  void add(void* p, size_t bytes) {
+    z.p[n] = (uint4*)p;
+    z.words[n] = (bytes + 15) / 16;
+    words += z.words[n++];
+  }
+  cudaError_t run(cudaStream_t st) {
+    g_prof.total_launches.fetch_add(1, std::memory_order_relaxed);
+    const size_t blocks = (words + 255) / 256;
+    zero_segs_kernel<<<(unsigned)(blocks < 4096 ? blocks : 4096), 256, 0, st>>>(z);
+    return cudaGetLastError();
+  }
+};
+
+// Host words of the calls in flight: the sort's plan and the control block's copy, in pinned mapped
+// memory (a copy to pageable memory takes 5 us longer, and the plan can be read while the ORP runs).
+// kHostSlots slots, allocated once (4 KiB); a call that finds none free works without.
+struct HostSlot {
+  HostPlan plan;
+  uint32_t pad[7];
+  Ctrl ctrl;
+};
+constexpr int kHostSlots = 12;
+struct HostSlots {
+  std::mutex mu;
+  HostSlot* base = nullptr;
+  bool tried = false;
+  uint32_t busy = 0, seq = 0;
+};
+HostSlots g_slots;
+struct SlotLease {
+  HostSlot* h = nullptr;
+  uint32_t seq = 0;
+  int i = -1;
+  bool clean = false;  // the stream has been synchronised: nothing writes the slot any more
+  SlotLease() {
+    std::lock_guard<std::mutex> g(g_slots.mu);
+    if (!g_slots.tried) {
+      g_slots.tried = true;
+      void* p = nullptr;
+      if (cudaHostAlloc(&p, kHostSlots * sizeof(HostSlot), cudaHostAllocPortable | cudaHostAllocMapped) == cudaSuccess)
+        g_slots.base = (HostSlot*)p;
+      else
+        (void)cudaGetLastError();
+    }
+    if (!g_slots.base) return;
+    for (int x = 0; x < kHostSlots; ++x)
+      if (!((g_slots.busy >> x) & 1u)) {
+        g_slots.busy |= 1u << x;
+        i = x;
+        h = g_slots.base + x;
+        seq = ++g_slots.seq ? g_slots.seq : ++g_slots.seq;
+        h->plan.seq = 0;
+        return;
+      }
+  }
+  ~SlotLease() {
+    if (i < 0 || !clean) return;  // a call that failed halfway may still have its plan kernel in flight
+    std::lock_guard<std::mutex> g(g_slots.mu);
+    g_slots.busy &= ~(1u << i);
+  }
+  // The next attempt's plan gets a number of its own (the stream has been synchronised).
+  void renew() {
+    clean = true;
+    if (!h) return;
+    std::lock_guard<std::mutex> g(g_slots.mu);
+    seq = ++g_slots.seq ? g_slots.seq : ++g_slots.seq;
+  }
+  // Waits until the plan kernel has published; false if the stream ended or failed without it.
+  bool wait(cudaStream_t st) const {
+    for (uint32_t spin = 1;; ++spin) {
+      if (__atomic_load_n(&h->plan.seq, __ATOMIC_ACQUIRE) == seq) return true;
+      if ((spin & 0xFFFu) == 0) {
+        const cudaError_t e = cudaStreamQuery(st);
+        if (e == cudaErrorNotReady) continue;
+        (void)cudaGetLastError();
+        return e == cudaSuccess && __atomic_load_n(&h->plan.seq, __ATOMIC_ACQUIRE) == seq;
+      }
+    }
+  }
+};
 // Folds the finished event pairs into the per-class totals (the stream has been synchronised).
 // A launch that returned at once (a constant digit; the LSD passes when the hybrid sort ran; a
 // hybrid stage its mode does not run) counts as a skipped radix pass.
@@ -342,7 +440,7 @@ bos_status make_plan(uint64_t n, const bos_params* p, bool sort, Plan* pl, uint3
       }
       pl->pass_k[bnp - 1] = bl;
       pl->pass_C[bnp - 1] = c_for(bl, true);
-      // The streaming kernels: orp_stream.cu takes the first and middle passes (5 to 8 levels each, no
+      // The streaming kernels: orp_stream.cu takes the first and middle passes (4 to 8 levels each, no
       // cluster), orp_last.cu or, beyond its tile, the cluster kernel the last one.
       const uint32_t kmin = orp_stream_min_k();
       uint32_t ksf = (p->flags & BOS_FLAG_NO_STREAM) ? 0u : orp_stream_max_k(pl->R, p->Z, true, kMaxSmem);
@@ -353,27 +451,80 @@ bos_status make_plan(uint64_t n, const bos_params* p, bool sort, Plan* pl, uint3
         ksm = p->k >= kmin && ksm ? (ksm < p->k ? ksm : p->k) : 0u;
         kt = kt < p->k ? kt : p->k;
       }
-      // the fewest passes; with the packed-tile last pass where it needs no more of them than the
-      // cluster one, and about the levels in the last pass that its kernel runs best
-      uint32_t sl = 0, snp = 0;
-      const uint32_t kb = kt < orp_last_best_k(pl->R, p->Z) ? kt : orp_last_best_k(pl->R, p->Z);
-      for (uint32_t np = 1; ksf && !sl && np < bnp && (np == 1 || ksm); ++np) {
-        auto fits = [&](uint32_t l) { return l < L && L - l >= np * kmin && L - l <= ksf + (np - 1) * ksm; };
-        for (uint32_t l = kb; l > 0 && !sl; --l)
-          if (fits(l)) sl = l;
-        for (uint32_t l = kb + 1; l <= kt && !sl; ++l)
-          if (fits(l)) sl = l;
-        pl->last_tile = sl > 0;
-        for (uint32_t l = 1; l < L && !sl; ++l)
-          if (fits(l) && c_for(l, true)) sl = l;
-        snp = np;
+      // The cheapest split of the levels by the kernels' measured times: a pass takes a launch and as
+      // many rounds of subproblems as the SMs need (so a small array takes fewer levels a pass, which
+      // gives more subproblems), with no more passes than the cluster plan.
+      const uint32_t kmins = p->k ? kmin : 4u;
+      const double fill = (double)n / ((double)B * p->Z);
+      auto pass_us = [&](uint32_t k, double sub_us) {
+        return 6.0 + (double)((B >> k) / kPlanSms + ((B >> k) % kPlanSms ? 1 : 0)) * sub_us;
+      };
+      double best_us = 1e30;
+      uint32_t bk[3] = {0, 0, 0}, bn = 0, sl = 0;
+      double us_f[kMaxStreamK + 1] = {}, us_m[kMaxStreamK + 1] = {};
+      for (uint32_t k = kmins; k <= kMaxStreamK && k < L; ++k) {
+        us_f[k] = pass_us(k, orp_stream_sub_us(p->Z, k, true, fill));
+        us_m[k] = pass_us(k, orp_stream_sub_us(p->Z, k, false, fill));
       }
-      if (sl) {
+      double us_l = 0;
+      auto consider = [&](const uint32_t* ks, uint32_t np, uint32_t l) {  // np streaming passes, then l levels
+        double us = us_l + us_f[ks[0]];
+        for (uint32_t x = 1; x < np; ++x) us += us_m[ks[x]];
+        if (us < best_us) {
+          best_us = us;
+          bn = np;
+          for (uint32_t x = 0; x < np; ++x) bk[x] = ks[x];
+          sl = l;
+        }
+      };
+      for (uint32_t l = 1; ksf && l <= kt && l < L; ++l) {
+        us_l = pass_us(l, orp_last_sub_us(pl->R, p->Z, l, fill));
+        for (uint32_t f = kmins; f <= ksf && f + l <= L; ++f) {
+          const uint32_t M = L - l - f;
+          if (M == 0 && bnp >= 2) consider(&f, 1, l);
+          if (M >= kmins && M <= ksm && bnp >= 3) {
+            const uint32_t ks[2] = {f, M};
+            consider(ks, 2, l);
+          }
+          for (uint32_t m = kmins; bnp >= 4 && m <= ksm && m + kmins <= M; ++m)
+            if (M - m <= ksm) {
+              const uint32_t ks[3] = {f, m, M - m};
+              consider(ks, 3, l);
+            }
+        }
+      }
+      // A small array may be quicker on the cluster passes, which spread one subproblem over C SMs.
+      // Measured, ORP of 2^20 16-byte records: Z = 512 170 us against 217, Z = 1024 184 against 307 (the
+      // estimate: 2 ns per slot of a CTA's share; the loads' prefix costs the tile pass about 8 us).
+      uint32_t snp_max = !bn ? bnp : (double)B * p->Z >= 5e8 ? bn : 0u;  // see below
+      if (bn && !p->k && p->Z >= 512 && n < (1u << 22)) {
+        double us = 0;
+        for (uint32_t x = 0; x < bnp; ++x) {
+          const uint64_t ctas = (B >> pl->pass_k[x]) * pl->pass_C[x];
+          us += 6.0 + (double)((ctas + kPlanSms - 1) / kPlanSms) *
+                          (2.0 + 0.002 * (double)((1u << pl->pass_k[x]) / pl->pass_C[x]) * p->Z);
+        }
+        if (us < best_us + 8.0) bn = snp_max = 0;
+      }
+      pl->last_tile = bn > 0;
+      // streaming passes before the cluster kernel's last one: where the tile's last pass does not do, and
+      // where it saves one of several long passes (2^30 16-byte records at Z = 1024)
+      uint32_t snp = bn;
+      for (uint32_t np = 1; ksf && np < snp_max && (np == 1 || ksm); ++np)
+        for (uint32_t l = 1; l < L; ++l)
+          if (L - l >= np * kmin && L - l <= ksf + (np - 1) * ksm && c_for(l, true)) {
+            pl->last_tile = false;
+            snp = np;
+            sl = l;
+            np = kMaxPasses;
+            break;
+          }
+      if (snp) {
         const uint32_t S = L - sl;
         pl->npass = snp + 1;
-        // balanced split of S levels over snp passes, the first at most ksf, the others ksm
+        // the chosen split, or (cluster last pass) a balanced one, the first pass at most ksf levels
         for (uint32_t x = 0; x < snp; ++x) {
-          pl->pass_k[x] = S / snp + (x < S % snp ? 1u : 0u);
+          pl->pass_k[x] = pl->last_tile ? bk[x] : S / snp + (x < S % snp ? 1u : 0u);
           pl->pass_C[x] = 1;
           pl->pass_stream[x] = true;
         }
@@ -593,25 +744,32 @@ bos_status run(const void* d_in, void* d_out, uint64_t n, const bos_params* p, v
     ha.ctrl = ctrl;
   }
 
+  SlotLease slot;
   for (uint32_t attempt = 0; attempt < max_attempts; ++attempt) {
-    BOS_CUDA(zero_async(ctrl, sizeof(Ctrl), st));
-    BOS_CUDA(zero_async(ws + pl.off_status, pl.orp_tiles * 8, st));
+    slot.clean = false;
+    Zeroer zero;
+    zero.add(ctrl, sizeof(Ctrl));
+    zero.add(ws + pl.off_status, pl.orp_tiles * 8);
     if (sort && !merge) {
-      BOS_CUDA(zero_async(ra.hist, pl.digits * 256 * 4, st));
-      BOS_CUDA(zero_async(ra.status, (pl.radix_tiles + (hybrid ? 256 : 0)) * 256 * 8, st));
+      zero.add(ra.hist, pl.digits * 256 * 4);
+      zero.add(ra.status, (pl.radix_tiles + (hybrid ? 256 : 0)) * 256 * 8);
+      if (hybrid) zero.add(ha.joint, 65536 * 4);
+    }
+    BOS_CUDA(zero.run(st));
+    if (sort && !merge) {
       int ev = prof_begin(st, kKHist, (double)n * pl.key_bytes);
-      if (hybrid) {
-        BOS_CUDA(zero_async(ha.joint, 65536 * 4, st));
-        BOS_CUDA(launch_hybrid(ha, pl.R, 0, st));
-      } else {
+      if (hybrid)
+        BOS_CUDA(launch_hybrid(ha, pl.R, 0, nullptr, st));
+      else
         BOS_CUDA(launch_radix_hist(ra, pl.R, st));
-      }
       prof_end(ev, st);
       ev = prof_begin(st, kKPrep, 0.0);
-      BOS_CUDA(launch_radix_prep(ra, pl.R, st));
       if (hybrid) {
-        BOS_CUDA(launch_hybrid(ha, pl.R, 1, st));
-        count_launches(1);  // the plan kernel, inside the prep event
+        ha.host = slot.h ? &slot.h->plan : nullptr;
+        ha.host_seq = slot.seq;
+        BOS_CUDA(launch_hybrid(ha, pl.R, 1, nullptr, st));
+      } else {
+        BOS_CUDA(launch_radix_prep(ra, pl.R, st));
       }
       prof_end(ev, st);
     }
@@ -709,22 +867,42 @@ bos_status run(const void* d_in, void* d_out, uint64_t n, const bos_params* p, v
       BOS_CUDA(launch_merge_sort(merge_first, d_out, ws + pl.off_tmp, n, pl.R, (uint64_t*)(ws + pl.off_rstatus), st,
                                  hooks));
     else if (sort) {
-      if (hybrid)  // each stage returns at once unless the plan's mode runs it
+      // The passes that the plan calls for. The plan was made from the input's keys before the ORP, so
+      // the host reads it while the ORP runs; without a host slot every stage is launched and those
+      // that the plan does not call for return at once.
+      uint32_t mode = 4, live = 0xFFFFFFFFu, list[kSortClasses];
+      for (uint32_t& c : list) c = 0xFFFFFFFFu;
+      if (hybrid && slot.h) {
+        if (!slot.wait(st)) return BOS_ERR_CUDA;
+        mode = slot.h->plan.mode;
+        live = slot.h->plan.live;
+        for (uint32_t c = 0; c < kSortClasses; ++c) list[c] = slot.h->plan.list[c];
+      }
+      if (hybrid && mode)
         for (int stage = 2; stage <= 4; ++stage) {
+          if (stage < 4 && mode < (uint32_t)stage) continue;  // the partitions of modes 2 and 3
           const int ev = prof_begin(st, stage == 4 ? kKLocal : kKMsd, 2.0 * n * pl.R, (uint32_t)stage);
-          BOS_CUDA(launch_hybrid(ha, pl.R, stage, st));
-          if (stage == 4) count_launches(6);  // one launch per range class and the fallback's
+          BOS_CUDA(launch_hybrid(ha, pl.R, stage, list, st));
+          if (stage == 4) {  // one launch per range class that has ranges, and the fallback's
+            uint64_t k = list[5] ? 1 : 0;
+            for (uint32_t c : list) k += c ? 1 : 0;
+            count_launches(k - 1);
+          }
           prof_end(ev, st);
         }
-      for (uint32_t d = 0; d < pl.digits; ++d) {  // skipped when the hybrid sort runs
-        const int ev = prof_begin(st, kKRadix, 2.0 * n * pl.R, d);
-        BOS_CUDA(launch_radix_pass(ra, pl.R, d, st));
-        prof_end(ev, st);
-      }
+      if (!hybrid || mode == 0 || mode == 4)
+        for (uint32_t d = 0; d < pl.digits; ++d) {
+          if (!((live >> d) & 1u)) continue;
+          const int ev = prof_begin(st, kKRadix, 2.0 * n * pl.R, d);
+          BOS_CUDA(launch_radix_pass(ra, pl.R, d, st));
+          prof_end(ev, st);
+        }
     }
-    Ctrl h{};
+    Ctrl hs{};
+    Ctrl& h = slot.h ? slot.h->ctrl : hs;
     BOS_CUDA(cudaMemcpyAsync(&h, ctrl, sizeof(Ctrl), cudaMemcpyDeviceToHost, st));
     BOS_CUDA(cudaStreamSynchronize(st));
+    slot.renew();
     if (g_prof.on) prof_collect(h.radix_live, h.sort_mode);
     if (info) {
       info->attempts = attempt + 1;

@@ -86,13 +86,14 @@ cudaError_t launch_orp_fast(const PassArgs& a, int mode, uint32_t C, uint32_t ma
 uint32_t orp_stream_smem_bytes(int R, uint32_t Z, uint32_t k, bool first);
 // Most levels a streaming pass holds in smem_limit bytes (0: the kernel cannot take this Z).
 uint32_t orp_stream_max_k(int R, uint32_t Z, bool first, uint32_t smem_limit);
-inline uint32_t orp_stream_min_k() { return 5; }
+inline uint32_t orp_stream_min_k() { return 5; }  // of a caller-given k; automatic plans go down to 4
+double orp_stream_sub_us(uint32_t Z, uint32_t k, bool first, double fill);  // planner: one subproblem on one SM
 cudaError_t launch_orp_stream(const PassArgs& a, bool first, cudaStream_t st, int R, bool trace);
 
 // LAST pass with known final loads and table (orp_last.cu): a.load, a.status and a.ord filled by
 // launch_perm_table. Z a multiple of 32, <= 2048; k <= orp_last_max_k.
 uint32_t orp_last_max_k(int R, uint32_t Z);  // 0: the kernel cannot take this Z
-uint32_t orp_last_best_k(int R, uint32_t Z);  // the k a plan gives it when the pass count allows
+double orp_last_sub_us(int R, uint32_t Z, uint32_t k, double fill);  // planner: one subproblem on one SM
 cudaError_t launch_orp_last(const PassArgs& a, cudaStream_t st, int R, bool trace);
 
 // The ORP with O(1) client storage (oblivious.cu, Section 4.1): bitonic-sort MergeSplits, one
@@ -148,13 +149,19 @@ uint64_t radix_tiles(uint64_t n, int R);
 // sort of every range of groups; falls back to the LSD passes (ctrl->sort_mode = 0) when a group
 // exceeds hybrid_cap(R) records. stage: 0 histogram (hist and joint), 1 plan, 2 partition by the
 // top varying digit, 3 partition by the next one inside every bucket, 4 the on-chip sort.
+constexpr uint32_t kSortClasses = 6;
+// What the plan kernel tells the host (mapped pinned memory): the host launches only the passes and the
+// range classes that the plan calls for. seq is written last.
+struct HostPlan {
+  uint32_t seq, mode, live, list[kSortClasses];
+};
 struct HybridArgs {
   const void* in;                   // histogram source (the ORP's input: the same multiset of keys)
   void* buf0;                       // final output
   void* buf1;                       // scratch of n records
   uint64_t n;
   uint32_t* hist;                   // [digits][256] digit counts (shared with the LSD path)
-  const unsigned long long* dbase;  // [digits][256] exclusive digit offsets (radix prep)
+  unsigned long long* dbase;        // [digits][256] exclusive digit offsets (written by the plan)
   uint32_t* joint;                  // [65536] counts of the top two digits
   unsigned long long* gstart;       // [65537] group starts
   uint32_t* rlist;                  // [65537] first group of every range
@@ -165,12 +172,15 @@ struct HybridArgs {
   unsigned long long* status;       // look-back words for radix_tiles(n) + 256 tiles
   unsigned char* scratch;           // hybrid_spill_bytes(n, R): one spill buffer per on-chip-sort CTA
   uint32_t local_ctas;              // = hybrid_local_ctas(n, R)
+  HostPlan* host;                   // null: the plan stays on the device
+  uint32_t host_seq;
   Ctrl* ctrl;
 };
 uint32_t hybrid_cap(int R);
 uint32_t hybrid_local_ctas(uint64_t n, int R);
 size_t hybrid_spill_bytes(uint64_t n, int R);
-cudaError_t launch_hybrid(const HybridArgs& a, int R, int stage, cudaStream_t st);
+// list (stage 4): ranges of every class (their launches are left out where there are none).
+cudaError_t launch_hybrid(const HybridArgs& a, int R, int stage, const uint32_t* list, cudaStream_t st);
 // Radix stages over many arrays in one launch (batched sort).
 struct BatchRadix {
   const RadixArgs* args;  // device: one entry per array

@@ -27,6 +27,8 @@
 //
 // A subproblem with more reals than the tile (the planner leaves 2.5 standard deviations) is run in
 // parts, each a run of its final buckets that fits, reading its input once per part.
+#include <cmath>
+
 #include "common.cuh"
 #include "internal.h"
 
@@ -50,8 +52,8 @@ struct LastLayout {
 
 inline uint32_t l_align(uint32_t x, uint32_t a) { return (x + a - 1) / a * a; }
 
-inline uint32_t isqrt_up(uint32_t x) {
-  uint32_t r = 0;
+inline uint32_t isqrt_up(uint32_t x) {  // the smallest r with r * r >= x
+  uint32_t r = (uint32_t)std::sqrt((double)x);
   while (r * r < x) ++r;
   return r;
 }
@@ -384,16 +386,13 @@ cudaError_t last_k(const PassArgs& a, cudaStream_t st) {
 
 }  // namespace
 
-// Largest k <= 4 that keeps the widest batches beside its tile. Measured, n = 2^26 16-byte records,
-// Z = 1024: k = 3 (two buckets a batch) 0.96 ms, k = 4 (one) 1.17 ms; n = 2^24, Z = 512 (k = 3..5 with
-// four, four and two buckets): 0.376, 0.281, 0.365 ms.
-uint32_t orp_last_best_k(int R, uint32_t Z) {
-  uint32_t best = 0;
-  for (uint32_t k = 1; k <= 4 && k <= orp_last_max_k(R, Z); ++k) {
-    const LastLayout l = last_layout(R, Z, k);
-    if ((2u << l.lub) * Z > kBatchSlots || (4u << l.lub) > (1u << k)) best = k;
-  }
-  return best;
+// Microseconds of one subproblem on one SM (fill: reals per slot). Measured: n = 2^26 16-byte records,
+// Z = 1024, k = 3 (four batches of two buckets): 8.9 us; k = 4 (sixteen of one): 21.9; n = 2^24, Z = 512,
+// k = 4 (four batches of four buckets): 10.4, k = 5 (sixteen of two): 27.
+double orp_last_sub_us(int R, uint32_t Z, uint32_t k, double fill) {
+  const LastLayout l = last_layout(R, Z, k);
+  const double slots = (double)(Z << l.lub);
+  return (double)((1u << k) >> l.lub) * (0.5 + 0.6 * slots / 1024.0) + 0.7 + 0.00045 * R / 16 * fill * Z * (1u << k);
 }
 
 uint32_t orp_last_max_k(int R, uint32_t Z) {

@@ -76,7 +76,7 @@ constexpr uint32_t kDone = (kBatchSlots + 256 * 7) / 8;  // most chunks a batch 
 constexpr uint32_t kAcc = 11;           // level counters per lane of the last warp
 constexpr uint32_t kZeroRecs = 4096, kZeroTags = 512;  // bytes of dummies in shared memory (bulk stores)
 constexpr uint32_t kMaxZ = 2048;
-constexpr uint32_t kMinK = 5, kMaxK = 8;
+constexpr uint32_t kMinK = 4, kMaxK = 8;
 static_assert(kSub <= (kListWords >> kMaxK), "the smallest round always fits the lists");
 static_assert((kListWords >> kMaxK) + kChunk - 1 <= (kRingSlots >> kMaxK), "a full list fits a ring");
 static_assert((kListWords >> kMinK) + kChunk - 1 <= (kRingSlots >> kMinK), "a full list fits a ring");
@@ -574,6 +574,14 @@ uint32_t orp_stream_max_k(int R, uint32_t Z, bool first, uint32_t smem_limit) {
   for (uint32_t k = kMinK; k <= kMaxK; ++k)
     if (stream_layout(R, Z, k, first).total <= smem_limit) best = k;
   return best;
+}
+
+// Microseconds of one subproblem on one SM (fill: reals per slot): about 2.4 per batch of 1024 reals
+// (n = 2^29, Z = 1024, k = 8: 128 batches in 300 us), 2.2 per batch of half as many (n = 2^20, Z = 512).
+double orp_stream_sub_us(uint32_t Z, uint32_t k, bool first, double fill) {
+  const uint32_t per = first ? Z / 2 : Z, most = first ? kBatchRecs : kBatchSlots;
+  const uint32_t ub = per * 4 <= most ? 4u : per * 2 <= most ? 2u : 1u;
+  return (double)(1u << k) / ub * (1.9 + 0.5 * ub * fill * Z / 1024.0) + 2.0;
 }
 
 cudaError_t launch_orp_stream(const PassArgs& a, bool first, cudaStream_t st, int R, bool trace) {

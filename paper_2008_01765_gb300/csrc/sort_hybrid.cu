@@ -41,7 +41,8 @@ constexpr uint32_t kTicketClass = 13;     // .. 18: one per range class
 // Range classes by size, each with its own list and launch: 0 one warp per range (registers); 1..4 the
 // bin sort with the records in shared memory, 128 to 1024 threads (8, 4, 2 and 1 CTAs per SM); 5 the bin
 // sort with the keys in shared memory (1024 threads).
-constexpr uint32_t kClasses = 6, kMidClass = 3;
+constexpr uint32_t kClasses = kSortClasses, kMidClass = 3;
+static_assert(kClasses == 6, "Bin<R, 0..5>");
 constexpr uint32_t kFull = 20;            // a range with a fuller bin is sorted by LSD passes
 
 constexpr uint32_t kMetaLeft = 3, kMetaList = 4;  // meta words: ranges left over; list starts [kClasses + 1]
@@ -164,17 +165,50 @@ __device__ __forceinline__ unsigned long long plan_scan(unsigned long long v, un
   return ex;
 }
 
+// The plan for the host, which launches only the kernels that it calls for: the words, then the
+// sequence number the host waits for.
+__device__ void publish_plan(HostPlan* h, uint32_t seq, uint32_t mode, uint32_t live, const uint32_t* list) {
+  if (!h) return;
+  volatile HostPlan* v = h;
+  v->mode = mode;
+  v->live = live;
+  for (uint32_t y = 0; y < kClasses; ++y) v->list[y] = list ? list[y] : 0u;
+  __threadfence_system();
+  v->seq = seq;
+}
+
 template <int R>
 __global__ void __launch_bounds__(kPlanThreads) sort_plan_kernel(HybridArgs a) {
   constexpr int D = RecT<R>::kDigits;
   constexpr uint32_t kCap = Local<R>::kCap;
-  __shared__ uint32_t s_max[8], s_jmax, s_mode, s_dA, s_dB;
+  __shared__ uint32_t s_max[8], s_jmax, s_live, s_mode, s_dA, s_dB;
+  __shared__ uint32_t s_list[kClasses];
   __shared__ unsigned long long s_w[32];
   const uint32_t tid = threadIdx.x;
   if (tid < 8) s_max[tid] = 0;
-  if (tid == 0) s_jmax = 0;
+  if (tid == 0) s_jmax = s_live = 0;
   __syncthreads();
-  for (uint32_t x = tid; x < D * 256; x += kPlanThreads) atomicMax(&s_max[x >> 8], a.hist[x]);
+  // every digit's exclusive offsets, its fullest value, and whether it varies (1024 threads: four
+  // digits at a time, eight warps each)
+  for (uint32_t x0 = 0; x0 < D * 256; x0 += kPlanThreads) {
+    const uint32_t x = x0 + tid, lane = tid & 31u, warp = tid >> 5;
+    const uint32_t c = a.hist[x];
+    uint32_t incl = c;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, incl, o);
+      if (lane >= (uint32_t)o) incl += y;
+    }
+    if (lane == 31) s_w[warp] = incl;
+    const uint32_t mx = __reduce_max_sync(0xFFFFFFFFu, c);
+    if (lane == 0) atomicMax(&s_max[x >> 8], mx);
+    __syncthreads();
+    uint32_t before = 0;
+    for (uint32_t w = warp & ~7u; w < warp; ++w) before += (uint32_t)s_w[w];
+    a.dbase[x] = before + incl - c;
+    __syncthreads();
+  }
+  if (tid < D && (uint64_t)s_max[tid] < a.n) atomicOr(&s_live, 1u << tid);
   uint32_t jm = 0;
   for (uint32_t x = tid; x < kGroups; x += kPlanThreads) jm = a.joint[x] > jm ? a.joint[x] : jm;
   atomicMax(&s_jmax, jm);
@@ -198,11 +232,15 @@ __global__ void __launch_bounds__(kPlanThreads) sort_plan_kernel(HybridArgs a) {
     a.meta[0] = mode;
     a.meta[1] = s_dA;
     a.meta[2] = s_dB;
+    a.ctrl->radix_live = s_live;
   }
   __syncthreads();
   const uint32_t mode = s_mode, dA = s_dA;
   if (mode == 0) {
-    if (tid == 0) a.ctrl->sort_mode = 0;
+    if (tid == 0) {
+      a.ctrl->sort_mode = 0;
+      publish_plan(a.host, a.host_seq, 0, s_live, nullptr);
+    }
     return;
   }
   // groups: the whole array (mode 1), the values of dA (mode 2), the (dA, dB) pairs (mode 3)
@@ -290,7 +328,10 @@ __global__ void __launch_bounds__(kPlanThreads) sort_plan_kernel(HybridArgs a) {
       unsigned long long tot = 0;
       const uint32_t w = __reduce_add_sync(0xFFFFFFFFu, nc[y]);
       at[y] = list + (uint32_t)__shfl_sync(0xFFFFFFFFu, plan_scan(lane == 0 ? w : 0ull, s_w, &tot), 0);
-      if (tid == 0) a.meta[kMetaList + y] = list;
+      if (tid == 0) {
+        a.meta[kMetaList + y] = list;
+        s_list[y] = (uint32_t)tot;
+      }
       list += (uint32_t)tot;
     }
     if (tid == 0) {
@@ -316,12 +357,15 @@ __global__ void __launch_bounds__(kPlanThreads) sort_plan_kernel(HybridArgs a) {
     if (tid == 0) a.first[256] = ttot;
   }
   __syncthreads();
-  if (tid == 0) a.ctrl->sort_mode = mode;
+  if (tid == 0) {
+    a.ctrl->sort_mode = mode;
+    publish_plan(a.host, a.host_seq, mode, s_live, s_list);
+  }
 }
 
 // ---- 3, 4. MSD partitions ---------------------------------------------------------------------
 // Persistent, like the LSD pass: CTAs take tiles by ticket, so a launch whose mode does not run
-// it costs one early return per CTA.
+// it (the host did not learn the mode in time) costs one early return per CTA.
 
 template <int R>
 __global__ void __launch_bounds__(kThreads, 2) msd1_kernel(HybridArgs a) {
@@ -1065,12 +1109,14 @@ __global__ void __launch_bounds__(Bin<R, CLS>::kT, Bin<R, CLS>::kCtas) bin_sort_
 }
 
 template <int R, int CLS>
-cudaError_t launch_bins(const HybridArgs& a, int sms, cudaStream_t st) {
+cudaError_t launch_bins(const HybridArgs& a, uint32_t count, int sms, cudaStream_t st) {
+  if (count == 0) return cudaSuccess;
   auto kern = bin_sort_kernel<R, CLS>;
   static_assert(Bin<R, CLS>::kCtas * (BinSmem<R, CLS>::total + 1024) <= 233472, "the CTAs of this class fit an SM");
   const cudaError_t e = set_smem_optin(kern);
   if (e != cudaSuccess) return e;
-  kern<<<(unsigned)(sms * Bin<R, CLS>::kCtas), Bin<R, CLS>::kT, BinSmem<R, CLS>::total, st>>>(a);
+  const uint32_t grid = (uint32_t)(sms * Bin<R, CLS>::kCtas);
+  kern<<<grid < count ? grid : count, Bin<R, CLS>::kT, BinSmem<R, CLS>::total, st>>>(a);
   return cudaGetLastError();
 }
 
@@ -1199,7 +1245,7 @@ int device_sms() {
 }
 
 template <int R>
-cudaError_t launch_r(const HybridArgs& a, int stage, cudaStream_t st) {
+cudaError_t launch_r(const HybridArgs& a, int stage, const uint32_t* list, cudaStream_t st) {
   constexpr int D = RecT<R>::kDigits;
   cudaError_t e = cudaSuccess;
   const int sms = device_sms();
@@ -1233,13 +1279,18 @@ cudaError_t launch_r(const HybridArgs& a, int stage, cudaStream_t st) {
       break;
     }
     default: {
-      local_small_kernel<R><<<(unsigned)sms * 8, kSThreads, 0, st>>>(a);
-      if ((e = cudaGetLastError()) != cudaSuccess) return e;
-      if ((e = launch_bins<R, 1>(a, sms, st)) != cudaSuccess) return e;
-      if ((e = launch_bins<R, 2>(a, sms, st)) != cudaSuccess) return e;
-      if ((e = launch_bins<R, 3>(a, sms, st)) != cudaSuccess) return e;
-      if ((e = launch_bins<R, 4>(a, sms, st)) != cudaSuccess) return e;
-      if ((e = launch_bins<R, 5>(a, sms, st)) != cudaSuccess) return e;
+      if (list[0]) {
+        const uint32_t need = (list[0] + kSThreads / 32 - 1) / (kSThreads / 32);
+        local_small_kernel<R><<<need < (uint32_t)sms * 8 ? need : (unsigned)sms * 8, kSThreads, 0, st>>>(a);
+        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+      }
+      if ((e = launch_bins<R, 1>(a, list[1], sms, st)) != cudaSuccess) return e;
+      if ((e = launch_bins<R, 2>(a, list[2], sms, st)) != cudaSuccess) return e;
+      if ((e = launch_bins<R, 3>(a, list[3], sms, st)) != cudaSuccess) return e;
+      if ((e = launch_bins<R, 4>(a, list[4], sms, st)) != cudaSuccess) return e;
+      if (list[5] == 0) break;
+      if ((e = launch_bins<R, 5>(a, list[5], sms, st)) != cudaSuccess) return e;
+      // only class 5 leaves ranges over
       const uint32_t smem = local_smem_bytes<R>();
       if ((e = cudaFuncSetAttribute(local_sort_kernel<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) !=
           cudaSuccess)
@@ -1267,9 +1318,9 @@ size_t hybrid_spill_bytes(uint64_t n, int R) {
 
 uint32_t hybrid_cap(int R) { return R == 8 ? Local<8>::kCap : Local<16>::kCap; }
 
-cudaError_t launch_hybrid(const HybridArgs& a, int R, int stage, cudaStream_t st) {
+cudaError_t launch_hybrid(const HybridArgs& a, int R, int stage, const uint32_t* list, cudaStream_t st) {
   if (a.n == 0) return cudaSuccess;
-  return R == 8 ? launch_r<8>(a, stage, st) : launch_r<16>(a, stage, st);
+  return R == 8 ? launch_r<8>(a, stage, list, st) : launch_r<16>(a, stage, list, st);
 }
 
 }  // namespace bos
