@@ -12,9 +12,13 @@
 //     counts m for every final bucket exactly as the LAST pass will (the label digit of every
 //     real); the table kernel sorts slots 0..m-1 and pads the row with 0xFFFF;
 //   * all slots (a single pass that draws the labels itself): slots 0..Z-1 sorted.
-// One warp sorts one final bucket with no block-wide barrier: it draws the keys, counts the top 8
-// bits of w0 into 256 bins of its own, scans them, places each slot in its bin, and puts each
-// slot at its bin's start plus its rank among the bin's few members (compared by (w0, w1, s)).
+// One warp sorts one final bucket with no block-wide barrier: it draws the keys, counts the top 9
+// bits of w0 into 512 bins of its own (16 bits each), scans them, places each slot in its bin, and
+// puts each slot at its bin's start plus its rank among the bin's few members (compared by
+// (w0, w1, s)).
+// Bound by issue (63 % of the cycles) at 24 warps per SM, which the 9 KB of a warp allow. n = 2^24,
+// Z = 1024: 150 us (167 with 256 bins). Fewer warps with the keys in bin order (12 KB each) took a third
+// longer, keys in registers (32 unrolled rows) missed the instruction cache and took 204 us.
 #include "common.cuh"
 #include "internal.h"
 
@@ -22,8 +26,9 @@ namespace bos {
 
 namespace {
 
-constexpr int kPBins = 256;        // bins: top 8 bits of w0
-constexpr int kShift = 24;
+constexpr int kPBins = 512;        // bins: top 9 bits of w0
+constexpr int kShift = 23;
+constexpr int kPWords = kPBins / 2;  // two 16-bit bins per word
 constexpr uint32_t kMaxK = 12;     // final buckets per LAST subproblem: at most 2^12
 
 // Slot s3 sorts before slot s2 (same bucket, base = b*Z, equal w0): smaller w1, or equal w1 and
@@ -35,9 +40,9 @@ __device__ __noinline__ bool tie_less(uint64_t base, uint32_t s3, uint32_t s2, u
 }
 
 // warps per CTA and shared memory: per warp Z keys (u32), Z placed slots and Z row entries (u16),
-// 256 bins
+// 512 bins
 __host__ __device__ inline uint32_t table_warps(uint32_t Z) { return Z <= 1024 ? 8u : (Z <= 2048 ? 4u : 2u); }
-__host__ __device__ inline uint32_t warp_bytes(uint32_t Z) { return Z * 8 + kPBins * 4; }
+__host__ __device__ inline uint32_t warp_bytes(uint32_t Z) { return Z * 8 + kPWords * 4; }
 uint32_t table_smem(uint32_t Z) { return table_warps(Z) * warp_bytes(Z); }
 
 constexpr int kLT = 256;     // threads of the load-count kernel
@@ -117,15 +122,15 @@ __global__ void __launch_bounds__(256, 3) perm_table_kernel(PermTableArgs a) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   unsigned char* wbase = smem + warp * warp_bytes(Z);
   uint32_t* key = reinterpret_cast<uint32_t*>(wbase);               // [Z] w0 of each slot
-  uint32_t* bins = key + Z;                                         // [kPBins] starts, then ends
-  uint16_t* placed = reinterpret_cast<uint16_t*>(bins + kPBins);    // [Z] slots grouped by bin
+  uint32_t* bins = key + Z;                                         // [kPWords] starts, then ends
+  uint16_t* placed = reinterpret_cast<uint16_t*>(bins + kPWords);   // [Z] slots grouped by bin
   uint16_t* row = placed + Z;                                       // [Z] the sorted row
   const bool tagged = a.tag != nullptr;
 
   for (uint64_t b = (uint64_t)blockIdx.x * W + warp; b < a.B; b += (uint64_t)gridDim.x * W) {
     const uint64_t base = (a.bucket0 + b) * Z;  // the keys' counters use the global bucket
     const uint32_t m = tagged ? min(a.load[b], Z) : Z;
-    for (int x = lane; x < kPBins; x += 32) bins[x] = 0;
+    for (int x = lane; x < kPWords; x += 32) bins[x] = 0;
     __syncwarp();
     // keys and bin counts (four independent Philox chains per lane per step)
     for (uint32_t s0 = lane; s0 < m; s0 += 128) {
@@ -137,18 +142,19 @@ __global__ void __launch_bounds__(256, 3) perm_table_kernel(PermTableArgs a) {
         const uint32_t s = s0 + c * 32;
         if (s < m) {
           key[s] = w[c];
-          atomicAdd(&bins[w[c] >> kShift], 1u);
+          atomicAdd(&bins[w[c] >> (kShift + 1)], 1u << (((w[c] >> kShift) & 1u) * 16));
         }
       }
     }
     __syncwarp();
-    {  // exclusive scan of the bins: eight consecutive bins per lane
-      uint32_t v[kPBins / 32], sum = 0;
+    {  // exclusive scan of the bins: eight consecutive words (sixteen bins) per lane
+      uint32_t v[kPWords / 32], sum = 0;
 #pragma unroll
-      for (int e = 0; e < kPBins / 32; ++e) {
-        v[e] = bins[lane * (kPBins / 32) + e];
-        sum += v[e];
+      for (int e = 0; e < kPWords / 32; ++e) {
+        v[e] = bins[lane * (kPWords / 32) + e];
+        sum += v[e];  // packed: both halves stay below 2^16
       }
+      sum = (sum & 0xFFFFu) + (sum >> 16);
       uint32_t incl = sum;
 #pragma unroll
       for (int o = 1; o < 32; o <<= 1) {
@@ -157,9 +163,9 @@ __global__ void __launch_bounds__(256, 3) perm_table_kernel(PermTableArgs a) {
       }
       uint32_t run = incl - sum;
 #pragma unroll
-      for (int e = 0; e < kPBins / 32; ++e) {
-        bins[lane * (kPBins / 32) + e] = run;
-        run += v[e];
+      for (int e = 0; e < kPWords / 32; ++e) {
+        bins[lane * (kPWords / 32) + e] = run | (run + (v[e] & 0xFFFFu)) << 16;
+        run += (v[e] & 0xFFFFu) + (v[e] >> 16);
       }
     }
     __syncwarp();
@@ -170,7 +176,8 @@ __global__ void __launch_bounds__(256, 3) perm_table_kernel(PermTableArgs a) {
 #pragma unroll
       for (int c = 0; c < 4; ++c) {
         const uint32_t s = s0 + c * 32;
-        p[c] = s < m ? atomicAdd(&bins[key[s] >> kShift], 1u) : 0u;
+        const uint32_t b = s < m ? key[s] >> kShift : 0u, h = (b & 1u) * 16;
+        p[c] = s < m ? (atomicAdd(&bins[b >> 1], 1u << h) >> h) & 0xFFFFu : 0u;
       }
 #pragma unroll
       for (int c = 0; c < 4; ++c)
@@ -185,8 +192,9 @@ __global__ void __launch_bounds__(256, 3) perm_table_kernel(PermTableArgs a) {
         const uint32_t s = s0 + c * 32;
         ks[c] = s < m ? key[s] : 0u;
         const uint32_t bin = ks[c] >> kShift;
-        start[c] = s < m && bin ? bins[bin - 1] : 0u;
-        end[c] = s < m ? bins[bin] : 0u;
+        const uint16_t* ends = reinterpret_cast<const uint16_t*>(bins);
+        start[c] = s < m && bin ? ends[bin - 1] : 0u;
+        end[c] = s < m ? ends[bin] : 0u;
         rank[c] = 0;
       }
 #pragma unroll
