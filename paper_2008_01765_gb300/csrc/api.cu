@@ -1,5 +1,6 @@
 // C ABI of libbos (declared in include/bos.h): argument checks, pass planning, workspace layout
 // and the attempt loop of Algorithm 3.1 (retry with a fresh attempt counter on overflow).
+#include <algorithm>
 #include <atomic>
 #include <cstring>
 #include <mutex>
@@ -940,6 +941,10 @@ struct BatchIn {
 struct BatchArr {
   Plan pl;
   bool sort = false;
+  // streaming passes and the packed-tile last pass (orp_stream.cu, orp_last.cu) instead of pl's: their
+  // levels (np passes), and the table and the loads in the data region
+  uint32_t np = 0, k[3] = {0, 0, 0}, lvl[3] = {0, 0, 0};
+  size_t ord_off = 0, load_off = 0;
   size_t zero_off = 0, data_off = 0;  // per-array regions
   size_t st_off = 0, hist_off = 0, rst_off = 0;                      // inside the zero region
   size_t rec_off[2] = {0, 0}, tag_off[2] = {0, 0}, tmp_off = 0, dbase_off = 0;  // data region
@@ -947,16 +952,45 @@ struct BatchArr {
 
 struct BatchLayout {
   std::vector<BatchArr> arr;
-  size_t ctrl_off = 0, zero_end = 0, desc_off = 0, desc_bytes = 0, data_off = 0, total = 0;
+  size_t ctrl_off = 0, zero_end = 0, desc_off = 0, desc_bytes = 0, data_off = 0, list_off = 0, total = 0;
+  uint32_t list_cap = 0;  // most ranges of all arrays' sorts
+  uint32_t pack = 0;      // records of a range of packed groups
   int R = 8;
   uint32_t maxpass = 0, digits = 4;
 };
+
+// The streaming plan of a batch's array of L levels: one first pass of up to 8 levels (two streaming passes
+// beyond 12 levels) and up to 4 in the last. A batch has subproblems enough for every SM, so the fewest
+// passes are the cheapest. np = 0: the one-CTA-per-subproblem passes (few levels, other bucket sizes).
+struct BatchStreamZ {  // what the kernels take of one bucket size
+  uint32_t Z = 0, kt = 0;
+};
+void batch_stream_plan(const bos_params& p, uint32_t L, BatchStreamZ* z, BatchArr* a) {
+  if (p.Z % 32 || L < 5 || p.k || (p.flags & (BOS_FLAG_GENERIC | BOS_FLAG_NO_STREAM))) return;
+  if (z->Z != p.Z) {
+    z->Z = p.Z;
+    z->kt = orp_last_max_k((int)p.rec_bytes, p.Z);
+    if (orp_stream_max_k((int)p.rec_bytes, p.Z, true, kMaxSmem) < kMaxStreamK ||
+        orp_stream_max_k((int)p.rec_bytes, p.Z, false, kMaxSmem) < kMaxStreamK)
+      z->kt = 0;
+  }
+  const uint32_t kt = z->kt;
+  if (!kt) return;
+  const uint32_t l = kt < 4 ? (kt < L - 4 ? kt : L - 4) : (L - 4 < 4 ? L - 4 : 4u), S = L - l;
+  if (S > 2 * kMaxStreamK) return;
+  a->np = S <= kMaxStreamK ? 2 : 3;
+  a->k[0] = S <= kMaxStreamK ? S : (S + 1) / 2;
+  if (a->np == 3) a->k[1] = S / 2;
+  a->k[a->np - 1] = l;
+  for (uint32_t x = 1; x < a->np; ++x) a->lvl[x] = a->lvl[x - 1] + a->k[x - 1];
+}
 
 bos_status batch_layout(const BatchIn& b, BatchLayout* L) {
   if (!b.off || (!b.seeds && b.num) || (!b.ops && b.num)) return BOS_ERR_INVALID;
   L->R = (int)b.base.rec_bytes;
   L->digits = b.base.key_bytes;
   L->arr.assign(b.num, BatchArr{});
+  BatchStreamZ zs;
   size_t off = 0;
   off += kBatchHeader;
   L->ctrl_off = off;
@@ -971,6 +1005,12 @@ bos_status batch_layout(const BatchIn& b, BatchLayout* L) {
     const bos_status s = make_plan(b.off[j + 1] - b.off[j], &p, a.sort, &a.pl);
     if (s != BOS_OK) return s;
     if (a.pl.npass > kBatchMaxPass) return BOS_ERR_INVALID;
+    if (a.pl.n) {
+      bos_params q = b.base;
+      q.Z = p.Z;
+      batch_stream_plan(q, a.pl.L, &zs, &a);
+    }
+    if (a.sort && a.pl.n) L->list_cap += batch_sort_ranges(a.pl.n, L->R);
     L->maxpass = a.pl.npass > L->maxpass ? a.pl.npass : L->maxpass;
     a.zero_off = off;
     a.st_off = off; off = align256(off + a.pl.B * 8);
@@ -982,8 +1022,13 @@ bos_status batch_layout(const BatchIn& b, BatchLayout* L) {
   L->zero_end = off;
   // descriptors: PassArgs for every (array, pass), RadixArgs per array, prefix arrays
   L->desc_off = off;
-  size_t dsz = 0;
-  for (uint32_t j = 0; j < b.num; ++j) dsz += L->arr[j].pl.npass * sizeof(PassArgs);
+  size_t dsz = 512;  // alignment between the tables
+  for (uint32_t j = 0; j < b.num; ++j) {
+    const BatchArr& a = L->arr[j];
+    dsz += a.pl.npass * sizeof(PassArgs);
+    for (uint32_t x = 0; x < a.np; ++x)
+      dsz += (x + 1 < a.np ? sizeof(BatchStream) : 2 * sizeof(BatchLast)) + 2 * (a.pl.B >> a.k[x]) * sizeof(uint2);
+  }
   dsz += (size_t)b.num * sizeof(RadixArgs);
   dsz += (size_t)(kBatchMaxPass * 4 + 2) * (b.num + 1) * sizeof(uint64_t);
   L->desc_bytes = align256(dsz);
@@ -998,29 +1043,45 @@ bos_status batch_layout(const BatchIn& b, BatchLayout* L) {
       a.rec_off[x] = off; off = align256(off + slots * L->R);
       a.tag_off[x] = off; off = align256(off + slots * 4);
     }
+    if (a.np) {
+      a.ord_off = off;  off = align256(off + slots * 2);
+      a.load_off = off; off = align256(off + a.pl.B * 4);
+    }
     if (a.sort) {
       a.tmp_off = off;   off = align256(off + a.pl.n * L->R);
       a.dbase_off = off; off = align256(off + L->digits * 256 * 8);
     }
   }
+  uint64_t sorted = 0;
+  for (const BatchArr& a : L->arr) sorted += a.sort ? a.pl.n : 0u;
+  L->pack = batch_sort_pack(sorted, L->R);
+  L->list_off = off;
+  off = align256(off + (size_t)(kSortClasses - 1) * L->list_cap * sizeof(uint4));
   L->total = off;
   return BOS_OK;
 }
 
-// One launch of the sequence: an ORP pass (index, mode) or a radix stage.
+// One launch of the sequence: an ORP pass, the tables, or a stage of the sort.
+enum BatchKind { kBPass, kBHist, kBDigit, kBStreamFirst, kBStreamMid, kBTable, kBLast, kBSort };
 struct BatchLaunch {
-  int kind;  // 0 = ORP pass, 1 = radix histogram, 2 = radix offsets, 3 = radix digit pass
-  int mode;
-  uint32_t digit, smem;
+  BatchKind kind;
+  int mode;              // kBPass: kModeFirst, kModeLast; kBSort: stage
+  uint32_t digit, smem;  // digit: kBDigit; the most levels (kBTable), the levels (kBLast)
   BatchPass bp;
   BatchRadix br;
+  // streaming passes, tables, last passes
+  const void* args = nullptr;
+  const uint2* units = nullptr;
+  uint32_t nunits = 0, max_Z = 0;
+  uint32_t* ticket = nullptr;
+  BatchSort bs{};
 };
 
 // Builds the launch sequence for the arrays in `sel` (attempt[j] each) and, when `desc` is not
 // null, the descriptor bytes to copy into the workspace's descriptor region.
 bos_status batch_build(const BatchIn& b, const BatchLayout& L, char* ws, const std::vector<uint32_t>& sel,
                        const std::vector<uint32_t>& attempt, std::vector<BatchLaunch>* launches,
-                       std::vector<char>* desc) {
+                       std::vector<char>* desc, size_t* used = nullptr) {
   launches->clear();
   if (desc) desc->assign(L.desc_bytes, 0);
   const Trace tr = trace_snapshot();  // the trace buffer the descriptors carry (debug)
@@ -1066,9 +1127,124 @@ bos_status batch_build(const BatchIn& b, const BatchLayout& L, char* ws, const s
     br.nblocks = acc;
     br.ticket = tickets + ticket_slot;
     ticket_slot += L.digits;
+    BatchSort bs{};
+    bs.br = br;
+    bs.list = (uint4*)(ws + L.list_off);
+    bs.cap = L.list_cap;
+    bs.P = L.pack;
+    for (uint32_t j : sorts) bs.max_n = L.arr[j].pl.n > bs.max_n ? L.arr[j].pl.n : bs.max_n;
+    bs.count = tickets + ticket_slot;
+    ticket_slot += 2 * (kSortClasses - 1);
+    bs.ticket = tickets + ticket_slot++;
+    auto sort_stage = [&](int stage) {
+      BatchLaunch l{kBSort, stage, 0, 0, BatchPass{}, BatchRadix{}};
+      l.bs = bs;
+      launches->push_back(l);
+    };
     if (!sorts.empty()) {
-      launches->push_back(BatchLaunch{1, 0, 0, 0, BatchPass{}, br});
-      launches->push_back(BatchLaunch{2, 0, 0, 0, BatchPass{}, br});
+      launches->push_back(BatchLaunch{kBHist, 0, 0, 0, BatchPass{}, br});
+      sort_stage(0);
+    }
+    // ---- arrays with streaming passes: first passes, middle passes, tables, last passes by level count ----
+    auto put = [&](const void* src, size_t bytes) -> size_t {  // descriptor bytes; their position
+      const size_t pos = (dpos + 15) & ~size_t(15);
+      if (desc && pos + bytes <= desc->size()) std::memcpy(desc->data() + pos, src, bytes);
+      dpos = pos + bytes;
+      return pos;
+    };
+    auto pass_args = [&](uint32_t j, uint32_t x) {  // pass x of array j's streaming plan
+      const BatchArr& a = L.arr[j];
+      PassArgs pa{};
+      const bool last = x + 1 == a.np;
+      const uint32_t src = (x + 1) & 1, dst = x & 1;
+      pa.in = (const char*)b.d_in + b.off[j] * R;
+      if (x) {
+        pa.in_rec = ws + a.rec_off[src];
+        pa.in_tag = (const uint32_t*)(ws + a.tag_off[src]);
+      }
+      if (!last) {
+        pa.out_rec = ws + a.rec_off[dst];
+        pa.out_tag = (uint32_t*)(ws + a.tag_off[dst]);
+      } else {
+        pa.out0 = (char*)b.d_out + b.off[j] * R;
+        pa.out1 = a.sort ? ws + a.tmp_off : pa.out0;
+        pa.out_sel = a.sort ? 1u : 0u;
+        pa.status = (unsigned long long*)(ws + a.st_off);
+        pa.ord = (const uint16_t*)(ws + a.ord_off);
+        pa.load = (const uint32_t*)(ws + a.load_off);
+      }
+      pa.n = a.pl.n;
+      pa.B = a.pl.B;
+      pa.Z = a.pl.Z;
+      pa.L = a.pl.L;
+      pa.i = a.lvl[x];
+      pa.k = a.k[x];
+      pa.attempt = attempt[j];
+      pa.seed = b.seeds[j];
+      pa.ctrl = (Ctrl*)(ws + L.ctrl_off + (size_t)j * sizeof(Ctrl));
+      pa.trace = tr;
+      pa.buf_in_rec = src ? kBufRecB : kBufRecA;
+      pa.buf_in_tag = src ? kBufTagB : kBufTagA;
+      pa.buf_out_rec = dst ? kBufRecB : kBufRecA;
+      pa.buf_out_tag = dst ? kBufTagB : kBufTagA;
+      return pa;
+    };
+    for (int stage = 0; stage < 2; ++stage) {  // 0: first passes, 1: middle passes
+      std::vector<uint32_t> js;
+      for (uint32_t j : sel)
+        if (L.arr[j].pl.n && (int)L.arr[j].np >= 2 + stage) js.push_back(j);
+      if (js.empty()) continue;
+      // the largest subproblems first: they would otherwise end alone
+      std::stable_sort(js.begin(), js.end(), [&](uint32_t x, uint32_t y) {
+        return (L.arr[x].pl.n >> (L.arr[x].pl.L - L.arr[x].k[stage])) > (L.arr[y].pl.n >> (L.arr[y].pl.L - L.arr[y].k[stage]));
+      });
+      std::vector<BatchStream> args;
+      std::vector<uint2> units;
+      uint32_t smem = 0;
+      for (uint32_t x = 0; x < js.size(); ++x) {
+        const BatchArr& a = L.arr[js[x]];
+        BatchStream s{pass_args(js[x], (uint32_t)stage), orp_stream_layout(R, a.pl.Z, a.k[stage], stage == 0)};
+        smem = s.lay.total > smem ? s.lay.total : smem;
+        args.push_back(s);
+        for (uint32_t q = 0; q < a.pl.B >> a.k[stage]; ++q) units.push_back(make_uint2(x, q));
+      }
+      BatchLaunch l{stage ? kBStreamMid : kBStreamFirst, 0, 0, smem, BatchPass{}, BatchRadix{}};
+      l.args = dev(put(args.data(), args.size() * sizeof(BatchStream)));
+      l.units = (const uint2*)dev(put(units.data(), units.size() * sizeof(uint2)));
+      l.nunits = (uint32_t)units.size();
+      launches->push_back(l);
+    }
+    {
+      std::vector<BatchLast> args;
+      std::vector<uint32_t> js;
+      std::vector<uint2> units;
+      uint32_t max_k = 0, max_Z = 0;
+      for (uint32_t j : sel)
+        if (L.arr[j].pl.n && L.arr[j].np) js.push_back(j);
+      for (uint32_t x = 0; x < js.size(); ++x) {
+        const BatchArr& a = L.arr[js[x]];
+        const uint32_t k = a.k[a.np - 1];
+        args.push_back(BatchLast{pass_args(js[x], a.np - 1), orp_last_layout(R, a.pl.Z, k)});
+        max_k = k > max_k ? k : max_k;
+        max_Z = a.pl.Z > max_Z ? a.pl.Z : max_Z;
+        for (uint32_t q = 0; q < a.pl.B >> k; ++q) units.push_back(make_uint2(x, q));
+      }
+      if (!js.empty()) {
+        const size_t apos = put(args.data(), args.size() * sizeof(BatchLast));
+        BatchLaunch l{kBTable, 0, max_k, 0, BatchPass{}, BatchRadix{}};
+        l.args = dev(apos);
+        l.units = (const uint2*)dev(put(units.data(), units.size() * sizeof(uint2)));
+        l.nunits = (uint32_t)units.size();
+        l.max_Z = max_Z;
+        l.ticket = tickets + ticket_slot++;
+        launches->push_back(l);
+        uint32_t smem = 0;
+        for (const BatchLast& s : args) smem = s.lay.total > smem ? s.lay.total : smem;
+        l.kind = kBLast;
+        l.smem = smem;
+        launches->push_back(l);
+      }
+      dpos = (dpos + 15) & ~size_t(15);
     }
     // the digit passes come after the ORP passes (pushed at the end)
     for (uint32_t p = 0; p < L.maxpass; ++p) {
@@ -1076,7 +1252,7 @@ bos_status batch_build(const BatchIn& b, const BatchLayout& L, char* ws, const s
         std::vector<uint32_t> js;
         for (uint32_t j : sel) {
           const BatchArr& a = L.arr[j];
-          if (a.pl.n == 0 || p >= a.pl.npass) continue;
+          if (a.pl.n == 0 || a.np || p >= a.pl.npass) continue;
           const int m = (p == 0 ? kModeFirst : 0) | (p + 1 == a.pl.npass ? kModeLast : 0);
           if (m == mode) js.push_back(j);
         }
@@ -1137,13 +1313,19 @@ bos_status batch_build(const BatchIn& b, const BatchLayout& L, char* ws, const s
         bp.nblocks = acc2;
         bp.ticket = tickets + ticket_slot++;
         if (ticket_slot * 4 > kBatchHeader) return BOS_ERR_INVALID;
-        launches->push_back(BatchLaunch{0, mode, 0, smem, bp, BatchRadix{}});
+        launches->push_back(BatchLaunch{kBPass, mode, 0, smem, bp, BatchRadix{}});
       }
     }
-    if (!sorts.empty())
-      for (uint32_t d = 0; d < L.digits; ++d) launches->push_back(BatchLaunch{3, 0, d, 0, BatchPass{}, br});
+    if (!sorts.empty()) {
+      sort_stage(1);
+      sort_stage(2);
+      // the LSD passes: run by the collect step for the arrays whose plans leave them their keys
+      for (uint32_t d = 0; d < L.digits; ++d) launches->push_back(BatchLaunch{kBDigit, 0, d, 0, BatchPass{}, br});
+    }
+    if (ticket_slot * 4 > kBatchHeader) return BOS_ERR_INVALID;
   }
   if (dpos > L.desc_bytes) return BOS_ERR_INVALID;
+  if (used) *used = dpos;
   return BOS_OK;
 }
 
@@ -1151,10 +1333,22 @@ bos_status batch_enqueue(const BatchLayout& L, char* ws, const std::vector<Batch
   BOS_CUDA(zero_async(ws, L.zero_end, st));
   const bool trace = trace_snapshot().buf != nullptr;
   for (const BatchLaunch& l : launches) {
-    if (l.kind == 0) {
-      BOS_CUDA(launch_orp_pass_batched(l.bp, l.mode, l.smem, st, L.R, trace));
-    } else {
-      BOS_CUDA(launch_radix_batched(l.br, L.R, l.kind - 1, l.digit, st));
+    switch (l.kind) {
+      case kBPass: BOS_CUDA(launch_orp_pass_batched(l.bp, l.mode, l.smem, st, L.R, trace)); break;
+      case kBHist: BOS_CUDA(launch_radix_batched(l.br, L.R, 0, 0, st)); break;
+      case kBDigit: break;
+      case kBStreamFirst:
+      case kBStreamMid:
+        BOS_CUDA(launch_orp_stream_batched((const BatchStream*)l.args, l.units, l.nunits, l.smem, l.kind == kBStreamFirst, st,
+                                           L.R, trace));
+        break;
+      case kBTable:
+        BOS_CUDA(launch_perm_table_batched((const BatchLast*)l.args, l.units, l.nunits, l.digit, l.max_Z, l.ticket, st, trace));
+        break;
+      case kBLast:
+        BOS_CUDA(launch_orp_last_batched((const BatchLast*)l.args, l.units, l.nunits, l.smem, st, L.R, trace));
+        break;
+      case kBSort: BOS_CUDA(launch_batch_sort(l.bs, L.R, l.mode, st)); break;
     }
   }
   return BOS_OK;
@@ -1174,12 +1368,14 @@ bos_status batch_check_in(const BatchIn& b, const BatchLayout& L, void* d_ws, si
 // Writes the descriptors of `sel` (synchronous copy from host memory).
 bos_status batch_prepare(const BatchIn& b, const BatchLayout& L, char* ws, const std::vector<uint32_t>& sel,
                          const std::vector<uint32_t>& attempt, std::vector<BatchLaunch>* launches,
-                         cudaStream_t st) {
+                         cudaStream_t st, bool wait = true) {
   std::vector<char> desc;
-  bos_status s = batch_build(b, L, ws, sel, attempt, launches, &desc);
+  size_t used = 0;
+  bos_status s = batch_build(b, L, ws, sel, attempt, launches, &desc, &used);
   if (s != BOS_OK) return s;
-  BOS_CUDA(cudaMemcpyAsync(ws + L.desc_off, desc.data(), desc.size(), cudaMemcpyHostToDevice, st));
-  BOS_CUDA(cudaStreamSynchronize(st));
+  // a copy from pageable memory has left the host buffer when the call returns
+  if (used) BOS_CUDA(cudaMemcpyAsync(ws + L.desc_off, desc.data(), used, cudaMemcpyHostToDevice, st));
+  if (wait) BOS_CUDA(cudaStreamSynchronize(st));
   return BOS_OK;
 }
 
@@ -1192,6 +1388,8 @@ std::vector<uint32_t> all_arrays(uint32_t num) {
 // After an enqueue: reads every array's flags; arrays that overflowed run again (as a smaller
 // batch) with the next attempt counter, up to max_attempts; then the descriptors of the full
 // batch (attempt 0) are written back so a captured graph stays valid.
+// Arrays whose plan left the keys to the LSD radix sort take its passes here, once the host has seen
+// which digits vary: most batches have none, and the passes' launches would return at once.
 bos_status batch_collect(const BatchIn& b, const BatchLayout& L, char* ws, cudaStream_t st, uint32_t* h_attempts) {
   const uint32_t max_attempts = b.base.max_attempts ? b.base.max_attempts : kDefaultAttempts;
   std::vector<uint32_t> attempt(b.num, 0);
@@ -1202,12 +1400,24 @@ bos_status batch_collect(const BatchIn& b, const BatchLayout& L, char* ws, cudaS
     if (b.num) BOS_CUDA(cudaMemcpyAsync(h.data(), ws + L.ctrl_off, b.num * sizeof(Ctrl), cudaMemcpyDeviceToHost, st));
     BOS_CUDA(cudaStreamSynchronize(st));
     std::vector<uint32_t> failed;
+    uint32_t lsd = 0;
     for (uint32_t j : sel) {
       if (L.arr[j].pl.n == 0) continue;
+      if (L.arr[j].sort && !h[j].overflow && !h[j].sort_mode) lsd |= h[j].radix_live;
       if (h[j].timeout) result = BOS_ERR_TIMEOUT;
+      if (h[j].bad) result = BOS_ERR_CUDA;
       if (h[j].overflow) failed.push_back(j);
     }
-    if (result != BOS_OK || failed.empty()) break;
+    if (result != BOS_OK) break;
+    if (lsd) {
+      std::vector<BatchLaunch> launches;
+      const bos_status s = batch_build(b, L, ws, sel, attempt, &launches, nullptr);
+      if (s != BOS_OK) return s;
+      for (const BatchLaunch& l : launches)
+        if (l.kind == kBDigit && ((lsd >> l.digit) & 1u)) BOS_CUDA(launch_radix_batched(l.br, L.R, 2, l.digit, st));
+      BOS_CUDA(cudaStreamSynchronize(st));
+    }
+    if (failed.empty()) break;
     for (uint32_t j : failed) attempt[j]++;
     bool exhausted = false;
     for (uint32_t j : failed) exhausted |= attempt[j] >= max_attempts;
@@ -1385,12 +1595,17 @@ bos_status bos_sort_batched(const void* d_in, void* d_out, const uint64_t* h_off
                             const uint64_t* h_seeds, const uint32_t* h_Z, const uint8_t* h_ops,
                             const bos_params* base, void* d_ws, size_t ws_bytes, void* stream,
                             uint32_t* h_attempts) {
-  bos_status s = bos_batched_prepare(d_in, d_out, h_offsets, num, h_seeds, h_Z, h_ops, base, d_ws, ws_bytes, stream);
+  if (!base) return BOS_ERR_INVALID;  // prepare, enqueue and collect over one layout
+  BatchIn b{d_in, d_out, h_offsets, num, h_seeds, h_Z, h_ops, *base};
+  BatchLayout L;
+  bos_status s = batch_layout(b, &L);
   if (s != BOS_OK) return s;
-  s = bos_batched_enqueue(d_in, d_out, h_offsets, num, h_seeds, h_Z, h_ops, base, d_ws, ws_bytes, stream);
+  if ((s = batch_check_in(b, L, d_ws, ws_bytes)) != BOS_OK) return s;
+  std::vector<BatchLaunch> launches;
+  s = batch_prepare(b, L, (char*)d_ws, all_arrays(num), std::vector<uint32_t>(num, 0), &launches, (cudaStream_t)stream, false);
   if (s != BOS_OK) return s;
-  return bos_batched_collect(d_in, d_out, h_offsets, num, h_seeds, h_Z, h_ops, base, d_ws, ws_bytes, stream,
-                             h_attempts);
+  if ((s = batch_enqueue(L, (char*)d_ws, launches, (cudaStream_t)stream)) != BOS_OK) return s;
+  return batch_collect(b, L, (char*)d_ws, (cudaStream_t)stream, h_attempts);
 }
 
 bos_status bos_shard_layout(uint64_t n, uint32_t G, const bos_params* p, bos_shard_layout_t* out) {

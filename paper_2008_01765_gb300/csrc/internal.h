@@ -81,6 +81,34 @@ int orp_fast_occupancy(int R, int mode, uint32_t Z, uint32_t k, uint32_t C);
 cudaError_t launch_orp_fast(const PassArgs& a, int mode, uint32_t C, uint32_t max_clusters, cudaStream_t st,
                             int R, bool trace);
 
+// Batched forms of the streaming, table and packed-tile kernels: one CTA per unit, a unit being
+// subproblem y of array x of the launch's argument list.
+struct StreamLayout {  // shared memory of the streaming pass (orp_stream.cu)
+  uint32_t ring_rec, ring_tag, list, stage, stage_bytes, zero, cf, acc, tail, done, misc, total;
+  uint32_t stages, lub;  // batches in flight; log2 of the input buckets (groups) per batch
+};
+struct LastLayout {  // shared memory of the packed-tile last pass (orp_last.cu)
+  uint32_t stage, stage_bytes, cnt, base, fill, misc, total;
+  uint32_t cap, stages, lub, stride;  // tile records, stages, log2 buckets per batch, u16 per row of counts
+};
+struct BatchStream {
+  PassArgs a;
+  StreamLayout lay;
+};
+struct BatchLast {
+  PassArgs a;
+  LastLayout lay;
+};
+StreamLayout orp_stream_layout(int R, uint32_t Z, uint32_t k, bool first);
+LastLayout orp_last_layout(int R, uint32_t Z, uint32_t k);
+cudaError_t launch_orp_stream_batched(const BatchStream* args, const uint2* units, uint32_t nunits, uint32_t smem,
+                                      bool first, cudaStream_t st, int R, bool trace);
+cudaError_t launch_orp_last_batched(const BatchLast* args, const uint2* units, uint32_t nunits, uint32_t smem,
+                                    cudaStream_t st, int R, bool trace);
+// final loads with their prefix (units in array order, taken by ticket), and the table rows
+cudaError_t launch_perm_table_batched(const BatchLast* args, const uint2* units, uint32_t nunits, uint32_t max_k,
+                                      uint32_t max_Z, uint32_t* ticket, cudaStream_t st, bool trace);
+
 // Streaming first / middle ORP pass (orp_stream.cu): one CTA per subproblem, input buckets
 // through a TMA ring, output chunks write-combined in shared memory; Z a multiple of 32, <= 2048.
 uint32_t orp_stream_smem_bytes(int R, uint32_t Z, uint32_t k, bool first);
@@ -191,6 +219,23 @@ struct BatchRadix {
 };
 // stage 0 = histograms, 1 = digit offsets, 2 = the pass of `digit`
 cudaError_t launch_radix_batched(const BatchRadix& br, int R, int stage, uint32_t digit, cudaStream_t st);
+// Batched hybrid sort (sort_hybrid.cu): every array's plan (digit offsets, its mode: kBatchOnChip, 2 or 0,
+// its ranges in the lists of classes 0..4), the partition of the arrays in mode 2, then one launch per
+// class. The ORP's last pass writes the output buffer in either mode (both count as even).
+constexpr uint32_t kBatchOnChip = 4;  // the array is one range, sorted in place
+struct BatchSort {
+  BatchRadix br;
+  uint4* list;        // [kSortClasses - 1][cap] ranges: array, first record, records, sorted in place
+  uint32_t cap;
+  uint32_t P;         // records of a range of packed groups, at most
+  uint64_t max_n;     // records of the largest array: classes beyond its size are not launched
+  uint32_t* count;    // [kSortClasses - 1] ranges listed (zeroed), then [kSortClasses - 1] taken (zeroed)
+  uint32_t* ticket;   // partition tiles (zeroed)
+};
+uint32_t batch_sort_ranges(uint64_t n, int R);  // most ranges of an array of n records
+uint32_t batch_sort_pack(uint64_t records, int R);  // P for a batch of that many records
+// stage 0: plans; 1: partition; 2: the range classes
+cudaError_t launch_batch_sort(const BatchSort& bs, int R, int stage, cudaStream_t st);
 cudaError_t launch_radix_hist(const RadixArgs& a, int R, cudaStream_t st);
 cudaError_t launch_radix_prep(const RadixArgs& a, int R, cudaStream_t st);
 cudaError_t launch_radix_pass(const RadixArgs& a, int R, uint32_t digit, cudaStream_t st);

@@ -45,11 +45,6 @@ constexpr uint32_t kMaxK = 5;        // one lane per digit
 constexpr uint32_t kMaxStages = 4;
 constexpr uint32_t kSmemLimit = 232448 - 1024;
 
-struct LastLayout {
-  uint32_t stage, stage_bytes, cnt, base, fill, misc, total;
-  uint32_t cap, stages, lub, stride;  // tile records, stages, log2 buckets per batch, u16 per row of counts
-};
-
 inline uint32_t l_align(uint32_t x, uint32_t a) { return (x + a - 1) / a * a; }
 
 inline uint32_t isqrt_up(uint32_t x) {  // the smallest r with r * r >= x
@@ -95,9 +90,10 @@ LastLayout last_layout(int R, uint32_t Z, uint32_t k) {
   return l;
 }
 
+// Subproblems q0, q0 + qstep, .. below nsub of one array.
 template <int R, int K, bool TRACE>
-__global__ void __launch_bounds__(kLThreads, 1) orp_last_kernel(const __grid_constant__ PassArgs a,
-                                                                const __grid_constant__ LastLayout lay) {
+__device__ __forceinline__ void orp_last_body(const PassArgs& a, const LastLayout& lay, const uint64_t q0,
+                                              const uint64_t nsub, const uint32_t qstep) {
   using Rec = typename RecT<R>::T;
   extern __shared__ __align__(128) unsigned char smem[];
   constexpr uint32_t k = K, D = 1u << k;
@@ -111,7 +107,6 @@ __global__ void __launch_bounds__(kLThreads, 1) orp_last_kernel(const __grid_con
 
   const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const bool worker = warp < kLW;
-  const uint64_t nsub = a.B >> k;
   const uint32_t lub = lay.lub, ub = 1u << lub, NB = D >> lub, nst = lay.stages;
   const uint32_t nslot = ub * Z, nrow = nslot / 32;
   const Rec* in_rec = reinterpret_cast<const Rec*>(a.in_rec);
@@ -159,7 +154,7 @@ __global__ void __launch_bounds__(kLThreads, 1) orp_last_kernel(const __grid_con
   // A pass over a subproblem's input serves the part [u0, u1) of its final buckets. The next pass is
   // another part of the same subproblem (rare) or the CTA's next subproblem; `ahead` batches, counted
   // from the current pass's first, have been requested, nst of them in flight (nst <= NB).
-  uint64_t q = blockIdx.x;
+  uint64_t q = q0;
   if (q >= nsub) return;  // (the grid never exceeds nsub)
   uint32_t sp = 0;              // subproblem parity
   uint32_t st = 0, ph = 0;      // stage and parity of the next batch
@@ -179,7 +174,7 @@ __global__ void __launch_bounds__(kLThreads, 1) orp_last_kernel(const __grid_con
     u1 = D;
     while (bs[u1] - bs[u0] > lay.cap) --u1;
     const bool ends = u1 == D;  // the subproblem's last part
-    const uint64_t qn = ends ? q + gridDim.x : q;  // the next pass's subproblem
+    const uint64_t qn = ends ? q + qstep : q;  // the next pass's subproblem
     uint32_t a1 = 0, a2 = 0, a3 = 0, a4 = 0;  // the last warp: reals per group of 2, 4, 8, 16 digits
 
     uint32_t dr[kItems];  // digit | rank inside the row << 8; 0xFFFFFFFF: dummy
@@ -356,6 +351,40 @@ __global__ void __launch_bounds__(kLThreads, 1) orp_last_kernel(const __grid_con
 }
 
 template <int R, int K, bool TRACE>
+__global__ void __launch_bounds__(kLThreads, 1) orp_last_kernel(const __grid_constant__ PassArgs a,
+                                                                const __grid_constant__ LastLayout lay) {
+  orp_last_body<R, K, TRACE>(a, lay, blockIdx.x, a.B >> K, gridDim.x);
+}
+
+// Many arrays: one CTA per unit, whatever its levels (one launch: a batch of small arrays has few
+// subproblems of each level count).
+template <int R, bool TRACE>
+__global__ void __launch_bounds__(kLThreads, 1) orp_last_batched_kernel(const BatchLast* args, const uint2* units) {
+  __shared__ BatchLast sa;
+  const uint2 un = units[blockIdx.x];
+  for (uint32_t x = threadIdx.x; x < sizeof(BatchLast) / 4; x += kLThreads)
+    reinterpret_cast<uint32_t*>(&sa)[x] = reinterpret_cast<const uint32_t*>(args + un.x)[x];
+  __syncthreads();
+  const uint64_t q = un.y;
+  switch (sa.a.k) {
+    case 1: orp_last_body<R, 1, TRACE>(sa.a, sa.lay, q, q + 1, 1); break;
+    case 2: orp_last_body<R, 2, TRACE>(sa.a, sa.lay, q, q + 1, 1); break;
+    case 3: orp_last_body<R, 3, TRACE>(sa.a, sa.lay, q, q + 1, 1); break;
+    case 4: orp_last_body<R, 4, TRACE>(sa.a, sa.lay, q, q + 1, 1); break;
+    default: orp_last_body<R, 5, TRACE>(sa.a, sa.lay, q, q + 1, 1); break;
+  }
+}
+
+template <int R, bool TRACE>
+cudaError_t last_batched(const BatchLast* args, const uint2* units, uint32_t nunits, uint32_t smem, cudaStream_t st) {
+  auto kern = orp_last_batched_kernel<R, TRACE>;
+  const cudaError_t e = set_smem_optin(kern);
+  if (e != cudaSuccess) return e;
+  kern<<<nunits, kLThreads, smem, st>>>(args, units);
+  return cudaGetLastError();
+}
+
+template <int R, int K, bool TRACE>
 cudaError_t last_launch(const PassArgs& a, cudaStream_t st) {
   const LastLayout lay = last_layout(R, a.Z, a.k);
   auto kern = orp_last_kernel<R, K, TRACE>;
@@ -401,6 +430,17 @@ uint32_t orp_last_max_k(int R, uint32_t Z) {
   for (uint32_t k = 1; k <= kMaxK; ++k)
     if (last_layout(R, Z, k).cap) best = k;
   return best;
+}
+
+LastLayout orp_last_layout(int R, uint32_t Z, uint32_t k) { return last_layout(R, Z, k); }
+
+cudaError_t launch_orp_last_batched(const BatchLast* args, const uint2* units, uint32_t nunits, uint32_t smem,
+                                    cudaStream_t st, int R, bool trace) {
+  if (nunits == 0) return cudaSuccess;
+  if (R == 8) return trace ? last_batched<8, true>(args, units, nunits, smem, st)
+                           : last_batched<8, false>(args, units, nunits, smem, st);
+  return trace ? last_batched<16, true>(args, units, nunits, smem, st)
+               : last_batched<16, false>(args, units, nunits, smem, st);
 }
 
 cudaError_t launch_orp_last(const PassArgs& a, cudaStream_t st, int R, bool trace) {

@@ -81,11 +81,6 @@ static_assert(kSub <= (kListWords >> kMaxK), "the smallest round always fits the
 static_assert((kListWords >> kMaxK) + kChunk - 1 <= (kRingSlots >> kMaxK), "a full list fits a ring");
 static_assert((kListWords >> kMinK) + kChunk - 1 <= (kRingSlots >> kMinK), "a full list fits a ring");
 
-struct StreamLayout {
-  uint32_t ring_rec, ring_tag, list, stage, stage_bytes, zero, cf, acc, tail, done, misc, total;
-  uint32_t stages, lub;  // batches in flight; log2 of the input buckets (groups) per batch
-};
-
 inline uint32_t st_align(uint32_t x, uint32_t a) { return (x + a - 1) / a * a; }
 
 inline StreamLayout stream_layout(int R, uint32_t Z, uint32_t k, bool first) {
@@ -123,9 +118,10 @@ inline StreamLayout stream_layout(int R, uint32_t Z, uint32_t k, bool first) {
   return l;
 }
 
+// Subproblems q0, q0 + qstep, .. (mysub of them) of one array.
 template <int R, bool FIRST, bool TRACE>
-__global__ void __launch_bounds__(kSThreads, 1) orp_stream_kernel(const __grid_constant__ PassArgs a,
-                                                                  const __grid_constant__ StreamLayout lay) {
+__device__ __forceinline__ void orp_stream_body(const PassArgs& a, const StreamLayout& lay, const uint64_t q0,
+                                                const uint32_t mysub, const uint32_t qstep) {
   using Rec = typename RecT<R>::T;
   constexpr uint32_t kItems = (FIRST ? kBatchRecs : kBatchSlots) / kST;  // slots per thread per batch
   extern __shared__ __align__(128) unsigned char smem[];
@@ -145,10 +141,8 @@ __global__ void __launch_bounds__(kSThreads, 1) orp_stream_kernel(const __grid_c
   const bool worker = warp < kSW;
   const uint32_t ring = kRingSlots >> k, cap = kListWords >> k;
   const uint32_t third = 11 - k;  // ring = 3 << third
-  const uint64_t nsub = a.B >> k;
   const uint32_t lub = lay.lub, ub = 1u << lub, NB = D >> lub;  // batches per subproblem
   const uint32_t nst = lay.stages;
-  const uint32_t mysub = blockIdx.x < nsub ? (uint32_t)((nsub - 1 - blockIdx.x) / gridDim.x) + 1 : 0;
   const uint32_t nbatch = mysub * NB;
   const Rec* in_first = reinterpret_cast<const Rec*>(a.in);
   const Rec* in_rec = reinterpret_cast<const Rec*>(a.in_rec);
@@ -303,7 +297,7 @@ __global__ void __launch_bounds__(kSThreads, 1) orp_stream_kernel(const __grid_c
   };
 
   if (tid == kST)  // the first nst batches (NB >= nst)
-    for (uint32_t x = 0; x < nst && x < nbatch; ++x) issue(blockIdx.x, x, x);
+    for (uint32_t x = 0; x < nst && x < nbatch; ++x) issue(q0, x, x);
 
   // The dummy chunks of subproblem qq's buckets s*ub .. s*ub + ub - 1 (the last warp): bulk stores of
   // dummies from shared memory, to the records or the tags. They are issued with batch s of the
@@ -328,7 +322,7 @@ __global__ void __launch_bounds__(kSThreads, 1) orp_stream_kernel(const __grid_c
   };
 
   // One iteration per round: a round is a whole batch, or a part of one while a batch is redone.
-  uint64_t q = blockIdx.x;
+  uint64_t q = q0;
   uint32_t g = 0, s = 0, st = 0, par = 0;  // batch g is batch s of subproblem q; its stage and the stage's parity
   uint32_t pb = 0;      // the round's buffer of lists, counts and fills
   uint32_t rlo = 0, sz = kBatchSlots;  // the round's first slot and size
@@ -365,9 +359,9 @@ __global__ void __launch_bounds__(kSThreads, 1) orp_stream_kernel(const __grid_c
       clear_lists(pb ^ 1);
       pend = false;
       s = 0;
-      q += gridDim.x;
-      orec += (uint64_t)gridDim.x * D * Z;
-      otag += (uint64_t)gridDim.x * D * Z;
+      q += qstep;
+      orec += (uint64_t)qstep * D * Z;
+      otag += (uint64_t)qstep * D * Z;
       __syncthreads();
     }
     unsigned char* stg = smem + lay.stage + st * lay.stage_bytes;
@@ -436,7 +430,7 @@ __global__ void __launch_bounds__(kSThreads, 1) orp_stream_kernel(const __grid_c
             full = true;
         }
     } else if (g >= NB && sz == kBatchSlots) {  // once per batch
-      write_tail(q - gridDim.x, s, false);
+      write_tail(q - qstep, s, false);
     }
     if (__syncthreads_or(full)) {
       // a list ran out of places: again with half the slots (kSub at the least, which always fit)
@@ -504,7 +498,7 @@ __global__ void __launch_bounds__(kSThreads, 1) orp_stream_kernel(const __grid_c
       levels(pb);
       if (rhi == nslot) {
         check(s);
-        if (g >= NB) write_tail(q - gridDim.x, s, true);
+        if (g >= NB) write_tail(q - qstep, s, true);
       }
     }
     __syncthreads();
@@ -519,7 +513,7 @@ __global__ void __launch_bounds__(kSThreads, 1) orp_stream_kernel(const __grid_c
     if (!worker) {
       if (lane == 0 && g + nst < nbatch) {
         const bool wrap = s + nst >= NB;
-        issue(wrap ? q + gridDim.x : q, wrap ? s + nst - NB : s + nst, st);
+        issue(wrap ? q + qstep : q, wrap ? s + nst - NB : s + nst, st);
       }
       check1(g & 1);
     }
@@ -532,14 +526,43 @@ __global__ void __launch_bounds__(kSThreads, 1) orp_stream_kernel(const __grid_c
       par ^= 1u;
     }
   }
-  if (!worker && nbatch) {
-    for (uint32_t x = 0; x < NB; ++x) {
+  if (nbatch) {  // the last subproblem's dummies: all warps
+    for (uint32_t x = warp; x < NB; x += kSThreads / 32) {
       write_tail(q, x, true);
       write_tail(q, x, false);
     }
     tma_store_wait_all();
   }
 }
+
+template <int R, bool FIRST, bool TRACE>
+__global__ void __launch_bounds__(kSThreads, 1) orp_stream_kernel(const __grid_constant__ PassArgs a,
+                                                                  const __grid_constant__ StreamLayout lay) {
+  const uint64_t nsub = a.B >> a.k;
+  if (blockIdx.x < nsub)
+    orp_stream_body<R, FIRST, TRACE>(a, lay, blockIdx.x, (uint32_t)((nsub - 1 - blockIdx.x) / gridDim.x) + 1, gridDim.x);
+}
+
+// Many arrays: one CTA per unit.
+template <int R, bool FIRST, bool TRACE>
+__global__ void __launch_bounds__(kSThreads, 1) orp_stream_batched_kernel(const BatchStream* args, const uint2* units) {
+  __shared__ BatchStream sa;
+  const uint2 un = units[blockIdx.x];
+  for (uint32_t x = threadIdx.x; x < sizeof(BatchStream) / 4; x += kSThreads)
+    reinterpret_cast<uint32_t*>(&sa)[x] = reinterpret_cast<const uint32_t*>(args + un.x)[x];
+  __syncthreads();
+  orp_stream_body<R, FIRST, TRACE>(sa.a, sa.lay, un.y, 1, 1);
+}
+
+template <int R, bool FIRST, bool TRACE>
+cudaError_t stream_batched(const BatchStream* args, const uint2* units, uint32_t nunits, uint32_t smem, cudaStream_t st) {
+  auto kern = orp_stream_batched_kernel<R, FIRST, TRACE>;
+  const cudaError_t e = set_smem_optin(kern);
+  if (e != cudaSuccess) return e;
+  kern<<<nunits, kSThreads, smem, st>>>(args, units);
+  return cudaGetLastError();
+}
+
 
 template <int R, bool FIRST, bool TRACE>
 cudaError_t stream_launch(const PassArgs& a, cudaStream_t st) {
@@ -582,6 +605,23 @@ double orp_stream_sub_us(uint32_t Z, uint32_t k, bool first, double fill) {
   const uint32_t per = first ? Z / 2 : Z, most = first ? kBatchRecs : kBatchSlots;
   const uint32_t ub = per * 4 <= most ? 4u : per * 2 <= most ? 2u : 1u;
   return (double)(1u << k) / ub * (1.9 + 0.5 * ub * fill * Z / 1024.0) + 2.0;
+}
+
+StreamLayout orp_stream_layout(int R, uint32_t Z, uint32_t k, bool first) { return stream_layout(R, Z, k, first); }
+
+cudaError_t launch_orp_stream_batched(const BatchStream* args, const uint2* units, uint32_t nunits, uint32_t smem,
+                                      bool first, cudaStream_t st, int R, bool trace) {
+  if (nunits == 0) return cudaSuccess;
+  if (R == 8) {
+    if (first) return trace ? stream_batched<8, true, true>(args, units, nunits, smem, st)
+                            : stream_batched<8, true, false>(args, units, nunits, smem, st);
+    return trace ? stream_batched<8, false, true>(args, units, nunits, smem, st)
+                 : stream_batched<8, false, false>(args, units, nunits, smem, st);
+  }
+  if (first) return trace ? stream_batched<16, true, true>(args, units, nunits, smem, st)
+                          : stream_batched<16, true, false>(args, units, nunits, smem, st);
+  return trace ? stream_batched<16, false, true>(args, units, nunits, smem, st)
+               : stream_batched<16, false, false>(args, units, nunits, smem, st);
 }
 
 cudaError_t launch_orp_stream(const PassArgs& a, bool first, cudaStream_t st, int R, bool trace) {

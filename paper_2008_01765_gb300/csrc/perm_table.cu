@@ -53,81 +53,125 @@ constexpr int kLUnroll = 8;  // 16-byte tag loads in flight per thread
 // equal to u, as the LAST pass counts them. With a.status, the subproblems are taken by ticket and
 // status[q] gets the inclusive prefix of their reals (loads above Z, an overflow, count as Z).
 template <bool TRACE>
-__global__ void __launch_bounds__(kLT) final_load_kernel(PermTableArgs a) {
+__device__ __forceinline__ void final_load_unit(const PermTableArgs& a, uint64_t q) {
   extern __shared__ __align__(16) unsigned char smem[];
-  __shared__ uint32_t q_s;
   uint32_t* mcnt = reinterpret_cast<uint32_t*>(smem);
   const uint32_t Z = a.Z, D = 1u << a.k, cpb = Z / 4;  // 16-byte chunks per input bucket
   const uint32_t shift = a.L - a.i - a.k;
-  const uint64_t units = a.B >> a.k;
   const int tid = threadIdx.x;
-  uint64_t q = blockIdx.x;
-  while (true) {
-    if (a.status && tid == 0) q_s = atomicAdd(a.ticket, 1u);
-    for (uint32_t x = tid; x < D; x += kLT) mcnt[x] = 0;
-    __syncthreads();
-    if (a.status) q = q_s;
-    if (q >= units) break;
-    const uint64_t t = q & ((1ull << a.i) - 1), G = q >> a.i;
-    if (TRACE && tid == 0)
-      for (uint32_t s = 0; s < D; ++s)
-        trace_log<TRACE>(a.trace, kRead, a.buf_tag, Z * 4, ((G << (a.i + a.k)) + ((uint64_t)s << a.i) + t) * Z * 4);
-    const uint32_t nchunk = D * cpb;
-    for (uint32_t c0 = tid; c0 < nchunk; c0 += kLT * kLUnroll) {
-      uint4 v[kLUnroll];
+  for (uint32_t x = tid; x < D; x += kLT) mcnt[x] = 0;
+  __syncthreads();
+  const uint64_t t = q & ((1ull << a.i) - 1), G = q >> a.i;
+  if (TRACE && tid == 0)
+    for (uint32_t s = 0; s < D; ++s)
+      trace_log<TRACE>(a.trace, kRead, a.buf_tag, Z * 4, ((G << (a.i + a.k)) + ((uint64_t)s << a.i) + t) * Z * 4);
+  const uint32_t nchunk = D * cpb;
+  for (uint32_t c0 = tid; c0 < nchunk; c0 += kLT * kLUnroll) {
+    uint4 v[kLUnroll];
 #pragma unroll
-      for (int e = 0; e < kLUnroll; ++e) {
-        const uint32_t c = c0 + e * kLT;
-        v[e] = make_uint4(kDummy, kDummy, kDummy, kDummy);
-        if (c < nchunk) {
-          const uint32_t s = c / cpb, off = c - s * cpb;
-          const uint64_t gb = (G << (a.i + a.k)) + ((uint64_t)s << a.i) + t;
-          v[e] = reinterpret_cast<const uint4*>(a.tag + gb * Z)[off];  // Z multiple of 32: aligned
-        }
-      }
-#pragma unroll
-      for (int e = 0; e < kLUnroll; ++e) {
-        const uint32_t w[4] = {v[e].x, v[e].y, v[e].z, v[e].w};
-#pragma unroll
-        for (int f = 0; f < 4; ++f)
-          if (w[f] != kDummy) atomicAdd(&mcnt[(w[f] >> shift) & (D - 1)], 1u);
+    for (int e = 0; e < kLUnroll; ++e) {
+      const uint32_t c = c0 + e * kLT;
+      v[e] = make_uint4(kDummy, kDummy, kDummy, kDummy);
+      if (c < nchunk) {
+        const uint32_t s = c / cpb, off = c - s * cpb;
+        const uint64_t gb = (G << (a.i + a.k)) + ((uint64_t)s << a.i) + t;
+        v[e] = reinterpret_cast<const uint4*>(a.tag + gb * Z)[off];  // Z multiple of 32: aligned
       }
     }
-    __syncthreads();
-    for (uint32_t x = tid; x < D; x += kLT) a.load[q * D + x] = mcnt[x];
-    if (a.status && tid < 32) {
-      uint32_t total = 0;
-      for (uint32_t x = tid; x < D; x += 32) total += min(mcnt[x], Z);
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) total += __shfl_xor_sync(0xFFFFFFFFu, total, o);
-      if (tid == 0) {
-        if (q == 0) {
-          if (!a.skip_publish) st_status(a.status, st_word(kStIncl, 0, total));
-        } else {
-          st_status(a.status + q, st_word(kStAgg, 0, total));
-          const unsigned long long pre = lookback_window<8>(a.status, q, 1, 0, a.ctrl);
-          st_status(a.status + q, st_word(kStIncl, 0, pre + total));
-        }
+    for (int e = 0; e < kLUnroll; ++e) {
+      const uint32_t w[4] = {v[e].x, v[e].y, v[e].z, v[e].w};
+#pragma unroll
+      for (int f = 0; f < 4; ++f)
+        if (w[f] != kDummy) atomicAdd(&mcnt[(w[f] >> shift) & (D - 1)], 1u);
+    }
+  }
+  __syncthreads();
+  for (uint32_t x = tid; x < D; x += kLT) a.load[q * D + x] = mcnt[x];
+  if (a.status && tid < 32) {
+    uint32_t total = 0;
+    for (uint32_t x = tid; x < D; x += 32) total += min(mcnt[x], Z);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) total += __shfl_xor_sync(0xFFFFFFFFu, total, o);
+    if (tid == 0) {
+      if (q == 0) {
+        if (!a.skip_publish) st_status(a.status, st_word(kStIncl, 0, total));
+      } else {
+        st_status(a.status + q, st_word(kStAgg, 0, total));
+        const unsigned long long pre = lookback_window<8>(a.status, q, 1, 0, a.ctrl);
+        st_status(a.status + q, st_word(kStIncl, 0, pre + total));
       }
     }
-    __syncthreads();  // mcnt is cleared for the next subproblem
-    q += gridDim.x;
   }
 }
 
 template <bool TRACE>
-__global__ void __launch_bounds__(256, 3) perm_table_kernel(PermTableArgs a) {
-  extern __shared__ __align__(16) unsigned char smem[];
-  const uint32_t Z = a.Z, W = table_warps(Z);
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  unsigned char* wbase = smem + warp * warp_bytes(Z);
+__global__ void __launch_bounds__(kLT) final_load_kernel(PermTableArgs a) {
+  __shared__ uint32_t q_s;
+  const uint64_t units = a.B >> a.k;
+  uint64_t q = blockIdx.x;
+  while (true) {
+    if (a.status) {
+      if (threadIdx.x == 0) q_s = atomicAdd(a.ticket, 1u);
+      __syncthreads();
+      q = q_s;
+    }
+    if (q >= units) break;
+    final_load_unit<TRACE>(a, q);
+    __syncthreads();  // the counts are cleared for the next subproblem
+    q += gridDim.x;
+  }
+}
+
+// The table's arguments of a batch's array.
+__device__ __forceinline__ PermTableArgs table_args(const PassArgs& p) {
+  PermTableArgs a{};
+  a.bucket0 = p.bucket0;
+  a.ord = const_cast<uint16_t*>(p.ord);
+  a.tag = p.in_tag;
+  a.load = const_cast<uint32_t*>(p.load);
+  a.B = p.B;
+  a.Z = p.Z;
+  a.attempt = p.attempt;
+  a.i = p.i;
+  a.k = p.k;
+  a.L = p.L;
+  a.buf_tag = p.buf_in_tag;
+  a.seed = p.seed;
+  a.trace = p.trace;
+  a.status = p.status;
+  a.ctrl = p.ctrl;
+  return a;
+}
+
+// Many arrays: units by ticket, in array order, so that every look-back predecessor has started.
+template <bool TRACE>
+__global__ void __launch_bounds__(kLT) final_load_batched_kernel(const BatchLast* args, const uint2* units, uint32_t nunits,
+                                                                 uint32_t* ticket) {
+  __shared__ uint32_t t_s;
+  while (true) {
+    if (threadIdx.x == 0) t_s = atomicAdd(ticket, 1u);
+    __syncthreads();
+    const uint32_t t = t_s;
+    if (t >= nunits) break;
+    const uint2 un = units[t];
+    final_load_unit<TRACE>(table_args(args[un.x].a), un.y);
+    __syncthreads();
+  }
+}
+
+// The row of final bucket b, sorted by one warp in its shared memory at wbase.
+template <bool TRACE>
+__device__ __forceinline__ void table_row(const PermTableArgs& a, uint64_t b, unsigned char* wbase) {
+  const uint32_t Z = a.Z;
+  const int lane = threadIdx.x & 31;
   uint32_t* key = reinterpret_cast<uint32_t*>(wbase);               // [Z] w0 of each slot
   uint32_t* bins = key + Z;                                         // [kPWords] starts, then ends
   uint16_t* placed = reinterpret_cast<uint16_t*>(bins + kPWords);   // [Z] slots grouped by bin
   uint16_t* row = placed + Z;                                       // [Z] the sorted row
   const bool tagged = a.tag != nullptr;
 
-  for (uint64_t b = (uint64_t)blockIdx.x * W + warp; b < a.B; b += (uint64_t)gridDim.x * W) {
+  {
     const uint64_t base = (a.bucket0 + b) * Z;  // the keys' counters use the global bucket
     const uint32_t m = tagged ? min(a.load[b], Z) : Z;
     for (int x = lane; x < kPWords; x += 32) bins[x] = 0;
@@ -220,6 +264,24 @@ __global__ void __launch_bounds__(256, 3) perm_table_kernel(PermTableArgs a) {
   }
 }
 
+template <bool TRACE>
+__global__ void __launch_bounds__(256, 3) perm_table_kernel(PermTableArgs a) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  const uint32_t W = table_warps(a.Z), warp = threadIdx.x >> 5;
+  for (uint64_t b = (uint64_t)blockIdx.x * W + warp; b < a.B; b += (uint64_t)gridDim.x * W)
+    table_row<TRACE>(a, b, smem + warp * warp_bytes(a.Z));
+}
+
+// Many arrays: a CTA per unit (the final buckets of one LAST subproblem).
+template <bool TRACE>
+__global__ void __launch_bounds__(256, 3) perm_table_batched_kernel(const BatchLast* args, const uint2* units, uint32_t stride) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  const uint2 un = units[blockIdx.x];
+  const PermTableArgs a = table_args(args[un.x].a);
+  const uint32_t D = 1u << a.k, W = blockDim.x >> 5, warp = threadIdx.x >> 5;
+  for (uint32_t u = warp; u < D; u += W) table_row<TRACE>(a, (uint64_t)un.y * D + u, smem + warp * stride);
+}
+
 }  // namespace
 
 template <bool TRACE>
@@ -245,6 +307,33 @@ cudaError_t perm_table_launch(const PermTableArgs& a, cudaStream_t st) {
   const uint64_t need = (a.B + W - 1) / W, want = (uint64_t)sms * (occ > 0 ? occ : 1);
   perm_table_kernel<TRACE><<<(unsigned)(need < want ? need : want), W * 32, sm, st>>>(a);
   return cudaGetLastError();
+}
+
+template <bool TRACE>
+static cudaError_t table_batched(const BatchLast* args, const uint2* units, uint32_t nunits, uint32_t max_k, uint32_t max_Z,
+                                 uint32_t* ticket, cudaStream_t st) {
+  int dev = 0, sms = 0, occ = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  if (e != cudaSuccess) return e;
+  const uint32_t sl = (1u << max_k) * 4;
+  if ((e = set_smem_optin(final_load_batched_kernel<TRACE>)) != cudaSuccess) return e;
+  if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, final_load_batched_kernel<TRACE>, kLT, sl)) != cudaSuccess)
+    return e;
+  const uint32_t want = (uint32_t)sms * (occ > 0 ? occ : 1);
+  final_load_batched_kernel<TRACE><<<nunits < want ? nunits : want, kLT, sl, st>>>(args, units, nunits, ticket);
+  if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  const uint32_t W = table_warps(max_Z), stride = warp_bytes(max_Z);
+  if ((e = set_smem_optin(perm_table_batched_kernel<TRACE>)) != cudaSuccess) return e;
+  perm_table_batched_kernel<TRACE><<<nunits, W * 32, W * stride, st>>>(args, units, stride);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_perm_table_batched(const BatchLast* args, const uint2* units, uint32_t nunits, uint32_t max_k,
+                                      uint32_t max_Z, uint32_t* ticket, cudaStream_t st, bool trace) {
+  if (nunits == 0) return cudaSuccess;
+  return trace ? table_batched<true>(args, units, nunits, max_k, max_Z, ticket, st)
+               : table_batched<false>(args, units, nunits, max_k, max_Z, ticket, st);
 }
 
 cudaError_t launch_perm_table(const PermTableArgs& a, cudaStream_t st, bool trace) {

@@ -131,25 +131,29 @@ __global__ void __launch_bounds__(kThreads, 2) radix_pass_kernel(RadixArgs a, ui
 }
 
 // Batched: tickets over all tiles of all arrays; ticket t is tile t - first[j] of array j, so
-// inside every array the tiles start in order (the look-back stops at the array's tile 0).
+// inside every array the tiles start in order (the look-back stops at the array's tile 0). Arrays that
+// another sort takes (sort_mode) and constant digits are passed over.
 template <int R>
 __global__ void __launch_bounds__(kThreads, 2) radix_pass_batched_kernel(BatchRadix br, uint32_t digit) {
   __shared__ unsigned long long t_s;
   __shared__ uint32_t j_s;
-  if (threadIdx.x == 0) {
-    const uint64_t t = atomicAdd(br.ticket + digit, 1u);
-    uint32_t lo = 0, hi = br.narr;
-    while (hi - lo > 1) {
-      const uint32_t mid = (lo + hi) >> 1;
-      if (br.first[mid] <= t) lo = mid; else hi = mid;
+  while (true) {
+    if (threadIdx.x == 0) {
+      const uint64_t t = atomicAdd(br.ticket + digit, 1u);
+      uint32_t lo = 0, hi = br.narr;
+      while (t < br.nblocks && hi - lo > 1) {
+        const uint32_t mid = (lo + hi) >> 1;
+        if (br.first[mid] <= t) lo = mid; else hi = mid;
+      }
+      j_s = t < br.nblocks ? lo : 0xFFFFFFFFu;
+      t_s = t - br.first[lo];
     }
-    j_s = lo;
-    t_s = t - br.first[lo];
+    __syncthreads();
+    if (j_s == 0xFFFFFFFFu) break;
+    const RadixArgs& a = br.args[j_s];
+    if (((a.ctrl->radix_live >> digit) & 1u) && !a.ctrl->sort_mode) radix_pass_body<R>(a, digit, t_s);
+    __syncthreads();
   }
-  __syncthreads();
-  const RadixArgs& a = br.args[j_s];
-  if (!((a.ctrl->radix_live >> digit) & 1u)) return;
-  radix_pass_body<R>(a, digit, t_s);
 }
 
 template <int R>
@@ -186,16 +190,21 @@ cudaError_t launch_radix_batched(const BatchRadix& br, int R, int stage, uint32_
       radix_prep_batched_kernel<16><<<br.narr * RecT<16>::kDigits, 256, 0, st>>>(br);
   } else {  // one digit pass over every array's tiles
     if (br.nblocks == 0) return cudaSuccess;
+    int dev = 0, sms = 0;
+    cudaError_t e0 = cudaGetDevice(&dev);
+    if (e0 == cudaSuccess) e0 = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e0 != cudaSuccess) return e0;
+    const unsigned grid = (unsigned)(br.nblocks < 2ull * sms ? br.nblocks : 2ull * sms);  // two CTAs per SM
     if (R == 8) {
       const uint32_t sm = pass_smem<8>();
       cudaError_t e = set_smem_optin(radix_pass_batched_kernel<8>);
       if (e != cudaSuccess) return e;
-      radix_pass_batched_kernel<8><<<(unsigned)br.nblocks, kThreads, sm, st>>>(br, digit);
+      radix_pass_batched_kernel<8><<<grid, kThreads, sm, st>>>(br, digit);
     } else {
       const uint32_t sm = pass_smem<16>();
       cudaError_t e = set_smem_optin(radix_pass_batched_kernel<16>);
       if (e != cudaSuccess) return e;
-      radix_pass_batched_kernel<16><<<(unsigned)br.nblocks, kThreads, sm, st>>>(br, digit);
+      radix_pass_batched_kernel<16><<<grid, kThreads, sm, st>>>(br, digit);
     }
   }
   return cudaGetLastError();

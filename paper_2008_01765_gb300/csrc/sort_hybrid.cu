@@ -808,8 +808,9 @@ struct BinSmem {
   static constexpr uint32_t total = wsum + 32 * 4 + 48;
 };
 
-template <int R, int CLS>
-__global__ void __launch_bounds__(Bin<R, CLS>::kT, Bin<R, CLS>::kCtas) bin_sort_kernel(HybridArgs a) {
+// BATCH: the ranges of many arrays (bs.list); else one array's, listed by its plan.
+template <int R, int CLS, bool BATCH>
+__global__ void __launch_bounds__(Bin<R, CLS>::kT, Bin<R, CLS>::kCtas) bin_sort_kernel(HybridArgs a, BatchSort bs) {
   using Rec = typename RecT<R>::T;
   using Key = typename RecT<R>::Key;
   using L = BinSmem<R, CLS>;
@@ -817,9 +818,16 @@ __global__ void __launch_bounds__(Bin<R, CLS>::kT, Bin<R, CLS>::kCtas) bin_sort_
   constexpr uint32_t kItems = (kMax + T - 1) / T;
   constexpr uint32_t kU = 4;  // loads in flight per thread
   constexpr bool kRecs = L::kRecs;
-  const uint32_t mode = a.ctrl->sort_mode;
-  if (mode == 0) return;
-  const uint32_t l0 = a.meta[kMetaList + CLS], nlist = a.meta[kMetaList + CLS + 1] - l0;
+  static_assert(kRecs || !BATCH, "a batch's plans list no ranges of class 5");
+  uint32_t mode = 0, l0 = 0, nlist = 0;
+  if constexpr (BATCH) {
+    nlist = bs.count[CLS];
+  } else {
+    mode = a.ctrl->sort_mode;
+    if (mode == 0) return;
+    l0 = a.meta[kMetaList + CLS];
+    nlist = a.meta[kMetaList + CLS + 1] - l0;
+  }
   if (blockIdx.x >= nlist) return;
   extern __shared__ __align__(16) unsigned char bsm[];
   Rec* SR = reinterpret_cast<Rec*>(bsm);                          // [kMax] records (classes 1..4)
@@ -831,8 +839,29 @@ __global__ void __launch_bounds__(Bin<R, CLS>::kT, Bin<R, CLS>::kCtas) bin_sort_
   unsigned long long* red = reinterpret_cast<unsigned long long*>(wsum + 32);  // smallest and largest key
   unsigned long long* bar = red + 2;
   uint32_t* next = reinterpret_cast<uint32_t*>(red + 3);  // the CTA's next range
-  const Rec* src = sort_buf<R>(a, mode, mode - 1);
-  Rec* dst = sort_buf<R>(a, mode, mode);
+  // range t: its records, their place in the sort's output, their count, its array's control block
+  auto range = [&](uint32_t t, const Rec*& in, Rec*& out, uint64_t& m, Ctrl*& ctrl) {
+    if constexpr (BATCH) {
+      const uint4 e = bs.list[CLS * bs.cap + t];
+      const RadixArgs& ra = bs.br.args[e.x];
+      in = reinterpret_cast<const Rec*>(e.w ? ra.buf0 : ra.buf1) + e.y;  // in place, or from the scratch buffer
+      out = reinterpret_cast<Rec*>(ra.buf0) + e.y;
+      m = e.z;
+      ctrl = ra.ctrl;
+    } else {
+      const uint32_t r = a.ridx[l0 + t];
+      const uint64_t lo = a.gstart[a.rlist[r]];
+      in = sort_buf<R>(a, mode, mode - 1) + lo;
+      out = sort_buf<R>(a, mode, mode) + lo;
+      m = a.gstart[a.rlist[r + 1]] - lo;
+      ctrl = a.ctrl;
+    }
+  };
+  uint32_t* ticket;
+  if constexpr (BATCH)
+    ticket = bs.count + (kClasses - 1) + CLS;
+  else
+    ticket = &a.ctrl->tickets[kTicketClass + CLS];
   const uint32_t tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5;
   if (kRecs && tid == 0) {
     mbar_init(smem_u32(bar), 1);
@@ -841,13 +870,13 @@ __global__ void __launch_bounds__(Bin<R, CLS>::kT, Bin<R, CLS>::kCtas) bin_sort_
   uint32_t ti = blockIdx.x, parity = 0;  // the first range is the block's own, later ones come by ticket
 
   while (true) {
-    const uint32_t r = a.ridx[l0 + ti];
-    const uint64_t lo = a.gstart[a.rlist[r]];
-    const uint64_t m64 = a.gstart[a.rlist[r + 1]] - lo;
+    const Rec* in;
+    Rec* out;
+    uint64_t m64;
+    Ctrl* ctrl;
+    range(ti, in, out, m64, ctrl);
     const bool fits = m64 > 0 && m64 <= kMax;  // always: the plan lists only this class's sizes
     const uint32_t m = fits ? (uint32_t)m64 : 0u;
-    const Rec* in = src + lo;
-    Rec* out = dst + lo;
     // 8-byte records on an odd address start one slot into the array, so that the bulk copy's both
     // ends are 16-byte aligned; the records at the odd ends are copied by threads
     const uint32_t odd = kRecs && R == 8 ? (uint32_t)((reinterpret_cast<uintptr_t>(in) >> 3) & 1u) : 0u;
@@ -857,10 +886,10 @@ __global__ void __launch_bounds__(Bin<R, CLS>::kT, Bin<R, CLS>::kCtas) bin_sort_
         mbar_expect_tx(smem_u32(bar), (c1 - c0) * R);
         if (c1 > c0) tma_load(smem_u32(SR + odd + c0), in + c0, (c1 - c0) * R, smem_u32(bar));
       }
-      if (!fits) atomicExch(&a.ctrl->bad, 1u);
+      if (!fits) atomicExch(&ctrl->bad, 1u);
       red[0] = ~0ull;
       red[1] = 0;
-      *next = gridDim.x + atomicAdd(&a.ctrl->tickets[kTicketClass + CLS], 1u);
+      *next = gridDim.x + atomicAdd(ticket, 1u);
     }
     const uint32_t lg = m > 1 ? 32u - (uint32_t)__clz(m - 1) : 0u, nb = lg < kBits ? (lg > 6 ? lg : 6u) : kBits;
     for (uint32_t x = tid; x < (1u << nb) / 8; x += T) reinterpret_cast<uint4*>(bins)[x] = make_uint4(0, 0, 0, 0);
@@ -871,15 +900,19 @@ __global__ void __launch_bounds__(Bin<R, CLS>::kT, Bin<R, CLS>::kCtas) bin_sort_
     __syncthreads();
     const uint32_t tn = *next;
     if (kRecs && tid == 0 && tn < nlist) {  // the next range on its way to L2
-      const uint32_t rn = a.ridx[l0 + tn];
-      const uint64_t ln = a.gstart[a.rlist[rn]], en = a.gstart[a.rlist[rn + 1]];
-      const uintptr_t p0 = reinterpret_cast<uintptr_t>(src + ln) & ~(uintptr_t)15;
-      const uint32_t nby = (uint32_t)((reinterpret_cast<uintptr_t>(src + en) - p0) & ~(uintptr_t)15);
+      const Rec* in2;
+      Rec* out2;
+      uint64_t m2;
+      Ctrl* ctrl2;
+      range(tn, in2, out2, m2, ctrl2);
+      const uintptr_t p0 = (reinterpret_cast<uintptr_t>(in2) + 15) & ~(uintptr_t)15;
+      const uintptr_t p1 = reinterpret_cast<uintptr_t>(in2 + m2) & ~(uintptr_t)15;
+      const uint32_t nby = p1 > p0 ? (uint32_t)(p1 - p0) : 0u;
       if (nby) asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p0), "r"(nby) : "memory");
     }
     // ---- the smallest and the largest key ----
     auto key_at = [&](uint32_t j) -> Key { return kRecs ? load_key<R>(SR + odd + j) : SK[j]; };
-    if (kRecs) mbar_wait(smem_u32(bar), parity, a.ctrl);
+    if (kRecs) mbar_wait(smem_u32(bar), parity, ctrl);
     parity ^= 1u;
     Key kmin = ~Key(0), kmax = Key(0);
     for (uint32_t j0 = tid; j0 < m; j0 += kU * T) {
@@ -973,7 +1006,7 @@ __global__ void __launch_bounds__(Bin<R, CLS>::kT, Bin<R, CLS>::kCtas) bin_sort_
       }
       const uint16_t* order = pl;  // positions in key order
       if (crowded && !kRecs) {  // the other kernel's range
-        if (tid == 0) a.joint[atomicAdd(&a.meta[kMetaLeft], 1u)] = r;
+        if (tid == 0) a.joint[atomicAdd(&a.meta[kMetaLeft], 1u)] = a.ridx[l0 + ti];
         order = nullptr;
       } else if (crowded) {
         // ---- LSD passes. Warp w owns the positions [w c, (w + 1) c) of the current order; its counts
@@ -1111,12 +1144,12 @@ __global__ void __launch_bounds__(Bin<R, CLS>::kT, Bin<R, CLS>::kCtas) bin_sort_
 template <int R, int CLS>
 cudaError_t launch_bins(const HybridArgs& a, uint32_t count, int sms, cudaStream_t st) {
   if (count == 0) return cudaSuccess;
-  auto kern = bin_sort_kernel<R, CLS>;
+  auto kern = bin_sort_kernel<R, CLS, false>;
   static_assert(Bin<R, CLS>::kCtas * (BinSmem<R, CLS>::total + 1024) <= 233472, "the CTAs of this class fit an SM");
   const cudaError_t e = set_smem_optin(kern);
   if (e != cudaSuccess) return e;
   const uint32_t grid = (uint32_t)(sms * Bin<R, CLS>::kCtas);
-  kern<<<grid < count ? grid : count, Bin<R, CLS>::kT, BinSmem<R, CLS>::total, st>>>(a);
+  kern<<<grid < count ? grid : count, Bin<R, CLS>::kT, BinSmem<R, CLS>::total, st>>>(a, BatchSort{});
   return cudaGetLastError();
 }
 
@@ -1200,11 +1233,28 @@ __device__ __forceinline__ void small_range(const typename RecT<R>::T* in, typen
     if (e < m) sidx[e] = (uint16_t)x[r];
   }
   __syncwarp();
-  for (uint32_t e = lane; e < m; e += 32) out[e] = in[sidx[e]];
+  typename RecT<R>::T v[EPL];  // all read before the first is written: out may be in
+#pragma unroll
+  for (int r = 0; r < EPL; ++r)
+    if ((uint32_t)r * 32 + lane < m) v[r] = in[sidx[r * 32 + lane]];
+  __syncwarp();
+#pragma unroll
+  for (int r = 0; r < EPL; ++r)
+    if ((uint32_t)r * 32 + lane < m) out[r * 32 + lane] = v[r];
   __syncwarp();
 }
 
 // The ranges of class 0 (many small groups), a warp each, taken by ticket; no block-wide barrier.
+template <int R>
+__device__ __forceinline__ void small_sort(const typename RecT<R>::T* in, typename RecT<R>::T* out, uint32_t m,
+                                           uint16_t* sidx, uint32_t lane) {
+  if (m == 0) return;
+  if (m <= 32) small_range<R, 1>(in, out, m, sidx, lane);
+  else if (m <= 64) small_range<R, 2>(in, out, m, sidx, lane);
+  else if (m <= 128) small_range<R, 4>(in, out, m, sidx, lane);
+  else small_range<R, 8>(in, out, m, sidx, lane);
+}
+
 template <int R>
 __global__ void __launch_bounds__(kSThreads) local_small_kernel(HybridArgs a) {
   using Rec = typename RecT<R>::T;
@@ -1228,13 +1278,133 @@ __global__ void __launch_bounds__(kSThreads) local_small_kernel(HybridArgs a) {
       if (lane == 0) atomicExch(&a.ctrl->bad, 1u);
       continue;
     }
-    const uint32_t m = (uint32_t)m64;
-    if (m == 0) continue;
-    if (m <= 32) small_range<R, 1>(src + lo, dst + lo, m, sidx[w], lane);
-    else if (m <= 64) small_range<R, 2>(src + lo, dst + lo, m, sidx[w], lane);
-    else if (m <= 128) small_range<R, 4>(src + lo, dst + lo, m, sidx[w], lane);
-    else small_range<R, 8>(src + lo, dst + lo, m, sidx[w], lane);
+    small_sort<R>(src + lo, dst + lo, (uint32_t)m64, sidx[w], lane);
   }
+}
+
+// ---- batched: the plans, the partition and the ranges of many arrays --------------------------
+
+// One CTA per array: the digit offsets, the live digits and the mode (kBatchOnChip: the array is one
+// range; 2: one partition by the top varying digit; 0: LSD passes), and the ranges into the lists of
+// their classes. Four digits at a time, eight warps each.
+template <int R>
+__global__ void __launch_bounds__(1024) batch_plan_kernel(BatchSort bs) {
+  constexpr uint32_t D = RecT<R>::kDigits, kCap = Bin<R, kClasses - 2>::kMax, kOne = Bin<R, 2>::kMax;
+  __shared__ uint32_t s_w[32], s_max[8], s_start[257], s_cnt[256], s_first[256];
+  const RadixArgs& a = bs.br.args[blockIdx.x];
+  const uint32_t tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5, n = (uint32_t)a.n;
+  if (tid < 8) s_max[tid] = 0;
+  __syncthreads();
+  for (uint32_t x = tid; x < D * 256; x += 1024) {
+    const uint32_t mx = __reduce_max_sync(0xFFFFFFFFu, a.hist[x]);
+    if (lane == 0) atomicMax(&s_max[x >> 8], mx);
+  }
+  __syncthreads();
+  uint32_t live = 0;
+  for (uint32_t d = 0; d < D; ++d) live |= s_max[d] < n ? 1u << d : 0u;  // some key differs in digit d
+  const uint32_t dA = live ? 31u - (uint32_t)__clz(live) : 0u;
+  for (uint32_t x = tid; x < D * 256; x += 1024) {
+    const uint32_t c = a.hist[x];
+    uint32_t incl = c;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, incl, o);
+      if (lane >= (uint32_t)o) incl += y;
+    }
+    if (lane == 31) s_w[warp] = incl;
+    __syncthreads();
+    uint32_t ex = incl - c;
+    for (uint32_t w = warp & ~7u; w < warp; ++w) ex += s_w[w];
+    a.dbase[x] = ex;
+    if (x >> 8 == dA) {
+      s_start[x & 255u] = ex;
+      s_cnt[x & 255u] = c;
+    }
+    __syncthreads();
+  }
+  const uint32_t maxA = s_max[dA];
+  const uint32_t mode = n < 2 || !live ? 0u : n <= kOne ? kBatchOnChip : maxA <= kCap ? 2u : 0u;
+  if (tid == 0) {
+    s_start[256] = n;
+    a.ctrl->radix_live = live;
+    a.ctrl->sort_mode = mode;
+  }
+  if (mode == 0) return;
+  auto list = [&](uint32_t lo, uint32_t m, uint32_t in_place) {
+    const uint32_t c = m <= Bin<R, 0>::kMax ? 0u : m <= Bin<R, 1>::kMax ? 1u : m <= Bin<R, 2>::kMax ? 2u
+                       : m <= Bin<R, 3>::kMax ? 3u : 4u;
+    bs.list[c * bs.cap + atomicAdd(&bs.count[c], 1u)] = make_uint4(blockIdx.x, lo, m, in_place);
+  };
+  if (mode == kBatchOnChip) {
+    if (tid == 0) list(0, n, 1);
+    return;
+  }
+  __syncthreads();
+  const bool single = maxA * 3 > bs.P;
+  const uint32_t S = single ? 1u : bs.P - maxA + 1u, v = tid & 255u, g = s_start[v];
+  const bool first = v == 0 || (single ? s_cnt[v] > 0 : g / S != (g - s_cnt[v - 1]) / S);
+  if (tid < 256) s_first[v] = first ? 1u : 0u;
+  __syncthreads();
+  if (tid < 256 && first) {
+    uint32_t e = v + 1;
+    while (e < 256 && !s_first[e]) ++e;
+    const uint32_t m = s_start[e] - g;
+    if (m) list(g, m, 0);
+  }
+}
+
+// The partition of the arrays in mode 2 (the top varying digit); tiles by ticket, in array order.
+template <int R>
+__global__ void __launch_bounds__(kThreads, 2) batch_msd_kernel(BatchSort bs) {
+  __shared__ unsigned long long t_s;
+  __shared__ uint32_t j_s;
+  while (true) {
+    if (threadIdx.x == 0) {
+      const uint64_t t = atomicAdd(bs.ticket, 1u);
+      uint32_t lo = 0, hi = bs.br.narr;
+      while (t < bs.br.nblocks && hi - lo > 1) {
+        const uint32_t mid = (lo + hi) >> 1;
+        if (bs.br.first[mid] <= t) lo = mid; else hi = mid;
+      }
+      j_s = t < bs.br.nblocks ? lo : 0xFFFFFFFFu;
+      t_s = t - bs.br.first[lo];
+    }
+    __syncthreads();
+    if (j_s == 0xFFFFFFFFu) break;
+    const RadixArgs& a = bs.br.args[j_s];
+    if (a.ctrl->sort_mode == 2) {
+      const uint32_t dA = 31u - (uint32_t)__clz(a.ctrl->radix_live);
+      radix_tile<R>(reinterpret_cast<const typename RecT<R>::T*>(a.buf0), reinterpret_cast<typename RecT<R>::T*>(a.buf1), a.n,
+                    t_s, 8 * dA, kTagMsd1, a.status, a.dbase + dA * 256, a.n, a.ctrl);
+    }
+    __syncthreads();
+  }
+}
+
+template <int R>
+__global__ void __launch_bounds__(kSThreads) batch_small_kernel(BatchSort bs) {
+  using Rec = typename RecT<R>::T;
+  __shared__ uint16_t sidx[kSThreads / 32][Bin<R, 0>::kMax];
+  const uint32_t lane = threadIdx.x & 31u, w = threadIdx.x >> 5, nlist = bs.count[0];
+  while (true) {
+    uint32_t t = 0;
+    if (lane == 0) t = atomicAdd(bs.count + kClasses - 1, 1u);
+    t = __shfl_sync(0xFFFFFFFFu, t, 0);
+    if (t >= nlist) break;
+    const uint4 e = bs.list[t];
+    const RadixArgs& a = bs.br.args[e.x];
+    small_sort<R>(reinterpret_cast<const Rec*>(e.w ? a.buf0 : a.buf1) + e.y, reinterpret_cast<Rec*>(a.buf0) + e.y, e.z, sidx[w], lane);
+  }
+}
+
+template <int R, int CLS>
+cudaError_t batch_bins(const BatchSort& bs, int sms, cudaStream_t st) {
+  auto kern = bin_sort_kernel<R, CLS, true>;
+  const cudaError_t e = set_smem_optin(kern);
+  if (e != cudaSuccess) return e;
+  const uint32_t grid = (uint32_t)(sms * Bin<R, CLS>::kCtas);
+  kern<<<grid < bs.cap ? grid : bs.cap, Bin<R, CLS>::kT, BinSmem<R, CLS>::total, st>>>(HybridArgs{}, bs);
+  return cudaGetLastError();
 }
 
 int device_sms() {
@@ -1303,7 +1473,43 @@ cudaError_t launch_r(const HybridArgs& a, int stage, const uint32_t* list, cudaS
   return cudaGetLastError();
 }
 
+template <int R>
+cudaError_t batch_sort_r(const BatchSort& bs, int stage, cudaStream_t st) {
+  const int sms = device_sms();
+  if (sms <= 0) return cudaErrorInvalidDevice;
+  cudaError_t e = cudaSuccess;
+  if (stage == 0) {
+    batch_plan_kernel<R><<<bs.br.narr, 1024, 0, st>>>(bs);
+  } else if (stage == 1) {
+    if ((e = set_smem_optin(batch_msd_kernel<R>)) != cudaSuccess) return e;
+    const uint64_t grid = bs.br.nblocks < 2ull * sms ? bs.br.nblocks : 2ull * sms;  // two CTAs per SM
+    batch_msd_kernel<R><<<(unsigned)grid, kThreads, radix_tile_smem<R>(), st>>>(bs);
+  } else {
+    batch_small_kernel<R><<<(unsigned)sms * 4, kSThreads, 0, st>>>(bs);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    if (bs.max_n > Bin<R, 0>::kMax && (e = batch_bins<R, 1>(bs, sms, st)) != cudaSuccess) return e;
+    if (bs.max_n > Bin<R, 1>::kMax && (e = batch_bins<R, 2>(bs, sms, st)) != cudaSuccess) return e;
+    if (bs.max_n > Bin<R, 2>::kMax && (e = batch_bins<R, 3>(bs, sms, st)) != cudaSuccess) return e;
+    if (bs.max_n > Bin<R, 3>::kMax && (e = batch_bins<R, 4>(bs, sms, st)) != cudaSuccess) return e;
+  }
+  return cudaGetLastError();
+}
+
 }  // namespace
+
+uint32_t batch_sort_ranges(uint64_t n, int) { return n <= Bin<16, 2>::kMax ? 1u : 256u; }
+static_assert(Bin<16, 2>::kMax == Bin<8, 2>::kMax, "one rule for both widths");
+
+// Ranges of class 1 (eight CTAs per SM) while the batch gives every SM few of them, then of class 3.
+uint32_t batch_sort_pack(uint64_t records, int R) {
+  if (records < (4u << 20)) return Bin<16, 1>::kMax;
+  return R == 8 ? Bin<8, kMidClass>::kMax : Bin<16, kMidClass>::kMax;
+}
+
+cudaError_t launch_batch_sort(const BatchSort& bs, int R, int stage, cudaStream_t st) {
+  if (bs.br.narr == 0 || bs.br.nblocks == 0) return cudaSuccess;
+  return R == 8 ? batch_sort_r<8>(bs, stage, st) : batch_sort_r<16>(bs, stage, st);
+}
 
 uint32_t hybrid_local_ctas(uint64_t n, int R) {
   const uint64_t cap = R == 8 ? Local<8>::kCap : Local<16>::kCap;
