@@ -115,7 +115,7 @@ __device__ __forceinline__ void radix_pass_body(const RadixArgs& a, uint32_t dig
 template <int R>
 // Persistent: CTAs take tiles by ticket until none is left (tiles start in ticket order, so every
 // look-back waits only on tiles already taken by running CTAs).
-__global__ void __launch_bounds__(kThreads, 2) radix_pass_kernel(RadixArgs a, uint32_t digit) {
+__global__ void __launch_bounds__(kTileThreads, 2) radix_pass_kernel(RadixArgs a, uint32_t digit) {
   __shared__ unsigned long long t_s;
   // a constant digit is skipped; so is every LSD pass when the hybrid sort runs instead
   if (!((a.ctrl->radix_live >> digit) & 1u) || a.ctrl->sort_mode) return;
@@ -134,7 +134,7 @@ __global__ void __launch_bounds__(kThreads, 2) radix_pass_kernel(RadixArgs a, ui
 // inside every array the tiles start in order (the look-back stops at the array's tile 0). Arrays that
 // another sort takes (sort_mode) and constant digits are passed over.
 template <int R>
-__global__ void __launch_bounds__(kThreads, 2) radix_pass_batched_kernel(BatchRadix br, uint32_t digit) {
+__global__ void __launch_bounds__(kTileThreads, 2) radix_pass_batched_kernel(BatchRadix br, uint32_t digit) {
   __shared__ unsigned long long t_s;
   __shared__ uint32_t j_s;
   while (true) {
@@ -199,12 +199,12 @@ cudaError_t launch_radix_batched(const BatchRadix& br, int R, int stage, uint32_
       const uint32_t sm = pass_smem<8>();
       cudaError_t e = set_smem_optin(radix_pass_batched_kernel<8>);
       if (e != cudaSuccess) return e;
-      radix_pass_batched_kernel<8><<<grid, kThreads, sm, st>>>(br, digit);
+      radix_pass_batched_kernel<8><<<grid, kTileThreads, sm, st>>>(br, digit);
     } else {
       const uint32_t sm = pass_smem<16>();
       cudaError_t e = set_smem_optin(radix_pass_batched_kernel<16>);
       if (e != cudaSuccess) return e;
-      radix_pass_batched_kernel<16><<<grid, kThreads, sm, st>>>(br, digit);
+      radix_pass_batched_kernel<16><<<grid, kTileThreads, sm, st>>>(br, digit);
     }
   }
   return cudaGetLastError();
@@ -230,12 +230,12 @@ cudaError_t launch_radix_pass(const RadixArgs& a, int R, uint32_t digit, cudaStr
     const uint32_t sm = pass_smem<8>();
     cudaError_t e = set_smem_optin(radix_pass_kernel<8>);
     if (e != cudaSuccess) return e;
-    radix_pass_kernel<8><<<grid, kThreads, sm, st>>>(a, digit);
+    radix_pass_kernel<8><<<grid, kTileThreads, sm, st>>>(a, digit);
   } else {
     const uint32_t sm = pass_smem<16>();
     cudaError_t e = set_smem_optin(radix_pass_kernel<16>);
     if (e != cudaSuccess) return e;
-    radix_pass_kernel<16><<<grid, kThreads, sm, st>>>(a, digit);
+    radix_pass_kernel<16><<<grid, kTileThreads, sm, st>>>(a, digit);
   }
   return cudaGetLastError();
 }

@@ -368,7 +368,7 @@ __global__ void __launch_bounds__(kPlanThreads) sort_plan_kernel(HybridArgs a) {
 // it (the host did not learn the mode in time) costs one early return per CTA.
 
 template <int R>
-__global__ void __launch_bounds__(kThreads, 2) msd1_kernel(HybridArgs a) {
+__global__ void __launch_bounds__(kTileThreads, 2) msd1_kernel(HybridArgs a) {
   const uint32_t mode = a.ctrl->sort_mode;
   if (mode < 2) return;
   __shared__ unsigned long long t_s;
@@ -386,7 +386,7 @@ __global__ void __launch_bounds__(kThreads, 2) msd1_kernel(HybridArgs a) {
 }
 
 template <int R>
-__global__ void __launch_bounds__(kThreads, 2) msd2_kernel(HybridArgs a) {
+__global__ void __launch_bounds__(kTileThreads, 2) msd2_kernel(HybridArgs a) {
   if (a.ctrl->sort_mode != 3) return;
   __shared__ unsigned long long t_s;
   __shared__ uint32_t b_s;
@@ -1355,7 +1355,7 @@ __global__ void __launch_bounds__(1024) batch_plan_kernel(BatchSort bs) {
 
 // The partition of the arrays in mode 2 (the top varying digit); tiles by ticket, in array order.
 template <int R>
-__global__ void __launch_bounds__(kThreads, 2) batch_msd_kernel(BatchSort bs) {
+__global__ void __launch_bounds__(kTileThreads, 2) batch_msd_kernel(BatchSort bs) {
   __shared__ unsigned long long t_s;
   __shared__ uint32_t j_s;
   while (true) {
@@ -1441,10 +1441,10 @@ cudaError_t launch_r(const HybridArgs& a, int stage, const uint32_t* list, cudaS
       const unsigned grid = (unsigned)(tiles < 2ull * sms ? tiles : 2ull * sms);  // two CTAs per SM
       if (stage == 2) {
         if ((e = set_smem_optin(msd1_kernel<R>)) != cudaSuccess) return e;
-        msd1_kernel<R><<<grid, kThreads, smem, st>>>(a);
+        msd1_kernel<R><<<grid, kTileThreads, smem, st>>>(a);
       } else {
         if ((e = set_smem_optin(msd2_kernel<R>)) != cudaSuccess) return e;
-        msd2_kernel<R><<<grid, kThreads, smem, st>>>(a);
+        msd2_kernel<R><<<grid, kTileThreads, smem, st>>>(a);
       }
       break;
     }
@@ -1483,7 +1483,7 @@ cudaError_t batch_sort_r(const BatchSort& bs, int stage, cudaStream_t st) {
   } else if (stage == 1) {
     if ((e = set_smem_optin(batch_msd_kernel<R>)) != cudaSuccess) return e;
     const uint64_t grid = bs.br.nblocks < 2ull * sms ? bs.br.nblocks : 2ull * sms;  // two CTAs per SM
-    batch_msd_kernel<R><<<(unsigned)grid, kThreads, radix_tile_smem<R>(), st>>>(bs);
+    batch_msd_kernel<R><<<(unsigned)grid, kTileThreads, radix_tile_smem<R>(), st>>>(bs);
   } else {
     batch_small_kernel<R><<<(unsigned)sms * 4, kSThreads, 0, st>>>(bs);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;

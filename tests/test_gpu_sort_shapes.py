@@ -61,6 +61,19 @@ def test_range_class_edges(bos, n, rec_bytes):
         np.testing.assert_array_equal(bos.to_host(out, recs.dtype), ref, err_msg=shape)
 
 
+# 4096-record tiles of a partition or LSD pass: the look-back's steps (7 single words, then one for eight
+# tiles, 64 tiles a window) and ragged last tiles
+@pytest.mark.parametrize("tiles,extra,rec_bytes", [(7, 0, 16), (7, 1, 8), (8, 1, 16), (9, -1, 16), (16, 0, 8), (63, 5, 16),
+                                                   (72, 31, 16), (73, 0, 8), (137, -33, 16)])
+def test_partition_tiles(bos, tiles, extra, rec_bytes):
+    n = 4096 * tiles + extra
+    for shape in ("uniform", "two", "low"):  # partitions; few and many values a digit in the LSD passes
+        recs = _keys(n, rec_bytes, shape, seed=n)
+        ref, _ = oracle.sort(recs, 512, 7, method=oracle.CLOSED)
+        out, _ = bos.sort(bos.to_device(recs), rec_bytes, Z=512, seed=7)
+        np.testing.assert_array_equal(bos.to_host(out, recs.dtype), ref, err_msg=shape)
+
+
 @pytest.mark.parametrize("n,rec_bytes,shape", [
     (200001, 16, "clusters"), (200001, 8, "clusters"), (1 << 20, 16, "span"), (300007, 8, "span"), (100003, 16, "extremes"),
     (100003, 8, "low"), ((1 << 23) + 1, 16, "clusters"), (1 << 23, 8, "clusters"),
