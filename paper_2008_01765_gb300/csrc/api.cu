@@ -865,7 +865,7 @@ bos_status run(const void* d_in, void* d_out, uint64_t n, const bos_params* p, v
       prof_end(ev, st);
     }
     if (merge)
-      BOS_CUDA(launch_merge_sort(merge_first, d_out, ws + pl.off_tmp, n, pl.R, (uint64_t*)(ws + pl.off_rstatus), st,
+      BOS_CUDA(launch_merge_sort(merge_first, d_out, ws + pl.off_tmp, n, pl.R, st,
                                  hooks));
     else if (sort) {
       // The passes that the plan calls for. The plan was made from the input's keys before the ORP, so

@@ -14,13 +14,6 @@ constexpr uint32_t kTile = kThreads * kItems;
 constexpr int kLook = 256;                      // look-back threads, one per digit value
 constexpr int kTileThreads = kThreads + kLook;  // of the kernels that run radix_tile
 
-template <int BYTES>
-__device__ __forceinline__ void cp_async(void* dst, const void* src) {
-  if constexpr (BYTES == 16)
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
-  else
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
-}
 template <int ID, int N>
 __device__ __forceinline__ void bar_sync() {
   asm volatile("bar.sync %0, %1;" ::"n"(ID), "n"(N) : "memory");

@@ -74,6 +74,17 @@ def test_partition_tiles(bos, tiles, extra, rec_bytes):
         np.testing.assert_array_equal(bos.to_host(out, recs.dtype), ref, err_msg=shape)
 
 
+# 4096-record runs and 2048-record chunks of the merge sort: ragged runs, lone left runs, ties across runs
+@pytest.mark.parametrize("n,rec_bytes", [(7, 16), (4095, 16), (4096, 8), (4097, 16), (8193, 8), (12287, 16), (14336, 16),
+                                         (65 * 4096 + 2049, 8), (65 * 4096 + 2049, 16)])
+def test_merge_runs(bos, n, rec_bytes):
+    for shape in ("uniform", "two", "equal", "extremes"):
+        recs = _keys(n, rec_bytes, shape, seed=n)
+        ref, _ = oracle.sort(recs, 512, 11, method=oracle.CLOSED)
+        out, _ = bos.sort(bos.to_device(recs), rec_bytes, Z=512, seed=11, flags=bos.FLAG_MERGE_SORT)
+        np.testing.assert_array_equal(bos.to_host(out, recs.dtype), ref, err_msg=shape)
+
+
 @pytest.mark.parametrize("n,rec_bytes,shape", [
     (200001, 16, "clusters"), (200001, 8, "clusters"), (1 << 20, 16, "span"), (300007, 8, "span"), (100003, 16, "extremes"),
     (100003, 8, "low"), ((1 << 23) + 1, 16, "clusters"), (1 << 23, 8, "clusters"),
