@@ -1414,7 +1414,7 @@ bos_status batch_collect(const BatchIn& b, const BatchLayout& L, char* ws, cudaS
       const bos_status s = batch_build(b, L, ws, sel, attempt, &launches, nullptr);
       if (s != BOS_OK) return s;
       for (const BatchLaunch& l : launches)
-        if (l.kind == kBDigit && ((lsd >> l.digit) & 1u)) BOS_CUDA(launch_radix_batched(l.br, L.R, 2, l.digit, st));
+        if (l.kind == kBDigit && ((lsd >> l.digit) & 1u)) BOS_CUDA(launch_radix_batched(l.br, L.R, 1, l.digit, st));
       BOS_CUDA(cudaStreamSynchronize(st));
     }
     if (failed.empty()) break;

@@ -161,32 +161,8 @@ __device__ __forceinline__ unsigned long long st_word(unsigned long long state, 
 
 // Exclusive prefix of tile `tile` over its predecessors (decoupled look-back, one thread). The
 // word of tile j is status[j * stride]. Spins with a limit; on timeout raises ctrl->timeout and
-// returns the prefix gathered so far.
-__device__ __forceinline__ unsigned long long lookback(const unsigned long long* status, uint64_t tile,
-                                                       uint64_t stride, uint32_t tag, Ctrl* ctrl) {
-  unsigned long long prefix = 0;
-  int64_t j = (int64_t)tile - 1;
-  while (j >= 0) {
-    unsigned long long w = 0;
-    uint32_t spins = 0;
-    while (true) {
-      w = ld_status(status + (uint64_t)j * stride);
-      if ((w >> 62) != 0 && ((w >> 56) & 63u) == tag) break;
-      if (++spins > kSpinLimit) {
-        atomicExch(&ctrl->timeout, 1u);
-        return prefix;
-      }
-      if (spins > 32) __nanosleep(64);
-    }
-    prefix += w & kStValue;
-    if (w & kStIncl) break;
-    --j;
-  }
-  return prefix;
-}
-
-// Windowed variant: each step issues the loads of W predecessors at once (independent loads, one
-// round-trip per W tiles), then folds them in order, waiting (bounded) on any not yet published.
+// returns the prefix gathered so far. Each step issues the loads of W predecessors at once
+// (independent loads, one round-trip per W tiles), then folds them in order, waiting (bounded) on any not yet published.
 template <int W>
 __device__ __forceinline__ unsigned long long lookback_window(const unsigned long long* status, uint64_t tile,
                                                               uint64_t stride, uint32_t tag, Ctrl* ctrl) {

@@ -216,7 +216,7 @@ struct BatchRadix {
   uint64_t nblocks;       // = first[narr]
   uint32_t* ticket;       // device: one zeroed counter per digit
 };
-// stage 0 = histograms, 1 = digit offsets, 2 = the pass of `digit`
+// stage 0 = histograms, 1 = the pass of `digit`
 cudaError_t launch_radix_batched(const BatchRadix& br, int R, int stage, uint32_t digit, cudaStream_t st);
 // Batched hybrid sort (sort_hybrid.cu): every array's plan (digit offsets, its mode: kBatchOnChip, 2 or 0,
 // its ranges in the lists of classes 0..4), the partition of the arrays in mode 2, then one launch per

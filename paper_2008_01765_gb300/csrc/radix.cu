@@ -66,7 +66,8 @@ __global__ void __launch_bounds__(kThreads) radix_hist_batched_kernel(BatchRadix
 }
 
 // Per digit: exclusive offsets of the 256 digit values, and whether the digit is live.
-__device__ __forceinline__ void radix_prep_body(const RadixArgs& a, int d) {
+__global__ void __launch_bounds__(256) radix_prep_kernel(RadixArgs a) {
+  const int d = blockIdx.x;
   __shared__ uint32_t s[256];
   __shared__ uint32_t any_full;
   const int v = threadIdx.x;
@@ -84,18 +85,6 @@ __device__ __forceinline__ void radix_prep_body(const RadixArgs& a, int d) {
   }
   a.dbase[d * 256 + v] = s[v] - c;
   if (v == 0 && !any_full) atomicOr(&a.ctrl->radix_live, 1u << d);
-}
-
-template <int R>
-__global__ void __launch_bounds__(256) radix_prep_kernel(RadixArgs a) {
-  radix_prep_body(a, blockIdx.x);
-}
-
-// Batched: block b = (array b / D, digit b % D).
-template <int R>
-__global__ void __launch_bounds__(256) radix_prep_batched_kernel(BatchRadix br) {
-  constexpr int D = RecT<R>::kDigits;
-  radix_prep_body(br.args[blockIdx.x / D], blockIdx.x % D);
 }
 
 // One tile of one live digit of the LSD chain (the whole CTA).
@@ -183,11 +172,6 @@ cudaError_t launch_radix_batched(const BatchRadix& br, int R, int stage, uint32_
       radix_hist_batched_kernel<8><<<(unsigned)br.nblocks, kThreads, 0, st>>>(br);
     else
       radix_hist_batched_kernel<16><<<(unsigned)br.nblocks, kThreads, 0, st>>>(br);
-  } else if (stage == 1) {  // digit offsets
-    if (R == 8)
-      radix_prep_batched_kernel<8><<<br.narr * RecT<8>::kDigits, 256, 0, st>>>(br);
-    else
-      radix_prep_batched_kernel<16><<<br.narr * RecT<16>::kDigits, 256, 0, st>>>(br);
   } else {  // one digit pass over every array's tiles
     if (br.nblocks == 0) return cudaSuccess;
     int dev = 0, sms = 0;
@@ -211,10 +195,7 @@ cudaError_t launch_radix_batched(const BatchRadix& br, int R, int stage, uint32_
 }
 
 cudaError_t launch_radix_prep(const RadixArgs& a, int R, cudaStream_t st) {
-  if (R == 8)
-    radix_prep_kernel<8><<<RecT<8>::kDigits, 256, 0, st>>>(a);
-  else
-    radix_prep_kernel<16><<<RecT<16>::kDigits, 256, 0, st>>>(a);
+  radix_prep_kernel<<<R == 8 ? RecT<8>::kDigits : RecT<16>::kDigits, 256, 0, st>>>(a);
   return cudaGetLastError();
 }
 
