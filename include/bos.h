@@ -167,15 +167,15 @@ bos_status bos_sort(const void* d_in, void* d_out, uint64_t n, const bos_params*
  * bos_sort of that array alone with the same seed and Z. h_attempts (nullable, num entries)
  * receives the attempts of each array (0 for an empty array). Host arrays are read during the
  * call only. All arrays go through one fixed sequence of launches (a reset, the key histograms and
- * the sorts' plans, the ORP passes, one partition, one launch per size class of the on-chip sort);
+ * the sorts' plans, the ORP passes, one partition, one launch per size class of the on-chip sort, one
+ * per radix digit for the arrays whose keys crowd one value of their top digit);
  * arrays that overflowed run again as a smaller batch with the next attempt counter.
  *
  * bos_sort_batched = bos_batched_prepare + bos_batched_enqueue + bos_batched_collect:
  *   - prepare writes the launch descriptors into d_ws (a synchronous copy);
  *   - enqueue only issues that launch sequence on `stream` (no copy, no synchronisation), so it
  *     can be captured into a CUDA graph and replayed for the same batch;
- *   - collect synchronises `stream`, reads every array's flags, runs the LSD radix passes of the
- *     arrays whose keys crowd one value of their top digit, reruns the arrays that
+ *   - collect synchronises `stream`, reads every array's overflow flag, reruns the arrays that
  *     overflowed and writes the full batch's descriptors back (so a captured graph stays valid).
  * The three calls take the same arguments (d_ws must be the same buffer). */
 size_t bos_batched_workspace_bytes(const uint64_t* h_offsets, uint32_t num, const uint32_t* h_Z,

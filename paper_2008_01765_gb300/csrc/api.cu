@@ -919,10 +919,9 @@ bos_status run(const void* d_in, void* d_out, uint64_t n, const bos_params* p, v
 }
 
 // ============================================================================================
-// Batched ORP / sort: many independent arrays through one fixed sequence of launches (one per
-// butterfly pass index and mode, one per radix stage), suitable for capture into a CUDA graph.
-// Every array uses the one-CTA-per-subproblem pass kernel; its plan, seed and Z are its own, so
-// its result equals bos_orp / bos_sort of that array alone.
+// Batched ORP / sort: many independent arrays through one fixed sequence of launches (one per pass
+// kernel, sort stage and size class of ranges), suitable for capture into a CUDA graph. Every array's
+// plan, seed and Z are its own, so its result equals bos_orp / bos_sort of that array alone.
 // ============================================================================================
 constexpr uint32_t kBatchMaxPass = 16;
 constexpr size_t kBatchHeader = 1024;  // launch tickets (zeroed with the control blocks)
@@ -1127,6 +1126,7 @@ bos_status batch_build(const BatchIn& b, const BatchLayout& L, char* ws, const s
     br.nblocks = acc;
     br.ticket = tickets + ticket_slot;
     ticket_slot += L.digits;
+    br.lsd = tickets + ticket_slot++;
     BatchSort bs{};
     bs.br = br;
     bs.list = (uint4*)(ws + L.list_off);
@@ -1319,8 +1319,11 @@ bos_status batch_build(const BatchIn& b, const BatchLayout& L, char* ws, const s
     if (!sorts.empty()) {
       sort_stage(1);
       sort_stage(2);
-      // the LSD passes: run by the collect step for the arrays whose plans leave them their keys
-      for (uint32_t d = 0; d < L.digits; ++d) launches->push_back(BatchLaunch{kBDigit, 0, d, 0, BatchPass{}, br});
+      // The LSD passes of the arrays whose keys crowd one value of their top digit: most batches have
+      // none, and each launch returns at once. Left out where every array fits a CTA's sort.
+      uint64_t max_n = 0;
+      for (uint32_t j : sorts) max_n = L.arr[j].pl.n > max_n ? L.arr[j].pl.n : max_n;
+      for (uint32_t d = 0; d < L.digits && max_n > batch_sort_cap(R); ++d) launches->push_back(BatchLaunch{kBDigit, 0, d, 0, BatchPass{}, br});
     }
     if (ticket_slot * 4 > kBatchHeader) return BOS_ERR_INVALID;
   }
@@ -1336,7 +1339,7 @@ bos_status batch_enqueue(const BatchLayout& L, char* ws, const std::vector<Batch
     switch (l.kind) {
       case kBPass: BOS_CUDA(launch_orp_pass_batched(l.bp, l.mode, l.smem, st, L.R, trace)); break;
       case kBHist: BOS_CUDA(launch_radix_batched(l.br, L.R, 0, 0, st)); break;
-      case kBDigit: break;
+      case kBDigit: BOS_CUDA(launch_radix_batched(l.br, L.R, 1, l.digit, st)); break;
       case kBStreamFirst:
       case kBStreamMid:
         BOS_CUDA(launch_orp_stream_batched((const BatchStream*)l.args, l.units, l.nunits, l.smem, l.kind == kBStreamFirst, st,
@@ -1388,8 +1391,6 @@ std::vector<uint32_t> all_arrays(uint32_t num) {
 // After an enqueue: reads every array's flags; arrays that overflowed run again (as a smaller
 // batch) with the next attempt counter, up to max_attempts; then the descriptors of the full
 // batch (attempt 0) are written back so a captured graph stays valid.
-// Arrays whose plan left the keys to the LSD radix sort take its passes here, once the host has seen
-// which digits vary: most batches have none, and the passes' launches would return at once.
 bos_status batch_collect(const BatchIn& b, const BatchLayout& L, char* ws, cudaStream_t st, uint32_t* h_attempts) {
   const uint32_t max_attempts = b.base.max_attempts ? b.base.max_attempts : kDefaultAttempts;
   std::vector<uint32_t> attempt(b.num, 0);
@@ -1400,23 +1401,13 @@ bos_status batch_collect(const BatchIn& b, const BatchLayout& L, char* ws, cudaS
     if (b.num) BOS_CUDA(cudaMemcpyAsync(h.data(), ws + L.ctrl_off, b.num * sizeof(Ctrl), cudaMemcpyDeviceToHost, st));
     BOS_CUDA(cudaStreamSynchronize(st));
     std::vector<uint32_t> failed;
-    uint32_t lsd = 0;
     for (uint32_t j : sel) {
       if (L.arr[j].pl.n == 0) continue;
-      if (L.arr[j].sort && !h[j].overflow && !h[j].sort_mode) lsd |= h[j].radix_live;
       if (h[j].timeout) result = BOS_ERR_TIMEOUT;
       if (h[j].bad) result = BOS_ERR_CUDA;
       if (h[j].overflow) failed.push_back(j);
     }
     if (result != BOS_OK) break;
-    if (lsd) {
-      std::vector<BatchLaunch> launches;
-      const bos_status s = batch_build(b, L, ws, sel, attempt, &launches, nullptr);
-      if (s != BOS_OK) return s;
-      for (const BatchLaunch& l : launches)
-        if (l.kind == kBDigit && ((lsd >> l.digit) & 1u)) BOS_CUDA(launch_radix_batched(l.br, L.R, 1, l.digit, st));
-      BOS_CUDA(cudaStreamSynchronize(st));
-    }
     if (failed.empty()) break;
     for (uint32_t j : failed) attempt[j]++;
     bool exhausted = false;

@@ -215,6 +215,7 @@ struct BatchRadix {
   uint32_t narr;
   uint64_t nblocks;       // = first[narr]
   uint32_t* ticket;       // device: one zeroed counter per digit
+  uint32_t* lsd;          // device: the digits that some array's LSD passes take (zeroed; set by the plans)
 };
 // stage 0 = histograms, 1 = the pass of `digit`
 cudaError_t launch_radix_batched(const BatchRadix& br, int R, int stage, uint32_t digit, cudaStream_t st);
@@ -232,6 +233,7 @@ struct BatchSort {
   uint32_t* ticket;   // partition tiles (zeroed)
 };
 uint32_t batch_sort_ranges(uint64_t n, int R);  // most ranges of an array of n records
+uint32_t batch_sort_cap(int R);                     // arrays above it may be left to the LSD passes
 uint32_t batch_sort_pack(uint64_t records, int R);  // P for a batch of that many records
 // stage 0: plans; 1: partition; 2: the range classes
 cudaError_t launch_batch_sort(const BatchSort& bs, int R, int stage, cudaStream_t st);

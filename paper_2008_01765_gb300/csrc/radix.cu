@@ -121,11 +121,13 @@ __global__ void __launch_bounds__(kTileThreads, 2) radix_pass_kernel(RadixArgs a
 
 // Batched: tickets over all tiles of all arrays; ticket t is tile t - first[j] of array j, so
 // inside every array the tiles start in order (the look-back stops at the array's tile 0). Arrays that
-// another sort takes (sort_mode) and constant digits are passed over.
+// another sort takes (sort_mode) and constant digits are passed over; a digit that no array's LSD passes
+// take ends the launch at once.
 template <int R>
 __global__ void __launch_bounds__(kTileThreads, 2) radix_pass_batched_kernel(BatchRadix br, uint32_t digit) {
   __shared__ unsigned long long t_s;
   __shared__ uint32_t j_s;
+  if (!((*br.lsd >> digit) & 1u)) return;
   while (true) {
     if (threadIdx.x == 0) {
       const uint64_t t = atomicAdd(br.ticket + digit, 1u);

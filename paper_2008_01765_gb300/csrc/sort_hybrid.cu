@@ -1328,6 +1328,7 @@ __global__ void __launch_bounds__(1024) batch_plan_kernel(BatchSort bs) {
     s_start[256] = n;
     a.ctrl->radix_live = live;
     a.ctrl->sort_mode = mode;
+    if (mode == 0 && live) atomicOr(bs.br.lsd, live);
   }
   if (mode == 0) return;
   auto list = [&](uint32_t lo, uint32_t m, uint32_t in_place) {
@@ -1521,6 +1522,8 @@ size_t hybrid_spill_bytes(uint64_t n, int R) {
   const size_t per = R == 8 ? (size_t)Local<8>::kCap * 6 : (size_t)Local<16>::kCap * 10;
   return per * hybrid_local_ctas(n, R);
 }
+
+uint32_t batch_sort_cap(int R) { return R == 8 ? Bin<8, kClasses - 2>::kMax : Bin<16, kClasses - 2>::kMax; }
 
 uint32_t hybrid_cap(int R) { return R == 8 ? Local<8>::kCap : Local<16>::kCap; }
 
