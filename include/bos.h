@@ -168,7 +168,7 @@ bos_status bos_sort(const void* d_in, void* d_out, uint64_t n, const bos_params*
  * receives the attempts of each array (0 for an empty array). Host arrays are read during the
  * call only. All arrays go through one fixed sequence of launches (a reset, the key histograms and
  * the sorts' plans, the ORP passes, one partition, one launch per size class of the on-chip sort, one
- * per radix digit for the arrays whose keys crowd one value of their top digit);
+ * of LSD radix passes for the arrays whose keys crowd one value of their top digit);
  * arrays that overflowed run again as a smaller batch with the next attempt counter.
  *
  * bos_sort_batched = bos_batched_prepare + bos_batched_enqueue + bos_batched_collect:

@@ -1061,11 +1061,11 @@ bos_status batch_layout(const BatchIn& b, BatchLayout* L) {
 }
 
 // One launch of the sequence: an ORP pass, the tables, or a stage of the sort.
-enum BatchKind { kBPass, kBHist, kBDigit, kBStreamFirst, kBStreamMid, kBTable, kBLast, kBSort };
+enum BatchKind { kBPass, kBHist, kBDigits, kBStreamFirst, kBStreamMid, kBTable, kBLast, kBSort };
 struct BatchLaunch {
   BatchKind kind;
   int mode;              // kBPass: kModeFirst, kModeLast; kBSort: stage
-  uint32_t digit, smem;  // digit: kBDigit; the most levels (kBTable), the levels (kBLast)
+  uint32_t digit, smem;  // digit: the most levels (kBTable), the levels (kBLast)
   BatchPass bp;
   BatchRadix br;
   // streaming passes, tables, last passes
@@ -1124,8 +1124,7 @@ bos_status batch_build(const BatchIn& b, const BatchLayout& L, char* ws, const s
     br.first = (const uint64_t*)dev(rfirst_pos);
     br.narr = (uint32_t)sorts.size();
     br.nblocks = acc;
-    br.ticket = tickets + ticket_slot;
-    ticket_slot += L.digits;
+    br.ticket = tickets + ticket_slot++;
     br.lsd = tickets + ticket_slot++;
     BatchSort bs{};
     bs.br = br;
@@ -1320,10 +1319,10 @@ bos_status batch_build(const BatchIn& b, const BatchLayout& L, char* ws, const s
       sort_stage(1);
       sort_stage(2);
       // The LSD passes of the arrays whose keys crowd one value of their top digit: most batches have
-      // none, and each launch returns at once. Left out where every array fits a CTA's sort.
+      // none, and the launch returns at once. Left out where every array fits a CTA's sort.
       uint64_t max_n = 0;
       for (uint32_t j : sorts) max_n = L.arr[j].pl.n > max_n ? L.arr[j].pl.n : max_n;
-      for (uint32_t d = 0; d < L.digits && max_n > batch_sort_cap(R); ++d) launches->push_back(BatchLaunch{kBDigit, 0, d, 0, BatchPass{}, br});
+      if (max_n > batch_sort_cap(R)) launches->push_back(BatchLaunch{kBDigits, 0, 0, 0, BatchPass{}, br});
     }
     if (ticket_slot * 4 > kBatchHeader) return BOS_ERR_INVALID;
   }
@@ -1338,8 +1337,8 @@ bos_status batch_enqueue(const BatchLayout& L, char* ws, const std::vector<Batch
   for (const BatchLaunch& l : launches) {
     switch (l.kind) {
       case kBPass: BOS_CUDA(launch_orp_pass_batched(l.bp, l.mode, l.smem, st, L.R, trace)); break;
-      case kBHist: BOS_CUDA(launch_radix_batched(l.br, L.R, 0, 0, st)); break;
-      case kBDigit: BOS_CUDA(launch_radix_batched(l.br, L.R, 1, l.digit, st)); break;
+      case kBHist: BOS_CUDA(launch_radix_batched(l.br, L.R, 0, st)); break;
+      case kBDigits: BOS_CUDA(launch_radix_batched(l.br, L.R, 1, st)); break;
       case kBStreamFirst:
       case kBStreamMid:
         BOS_CUDA(launch_orp_stream_batched((const BatchStream*)l.args, l.units, l.nunits, l.smem, l.kind == kBStreamFirst, st,

@@ -214,11 +214,11 @@ struct BatchRadix {
   const uint64_t* first;  // device: running sum of tiles (kTile records each), narr + 1 entries
   uint32_t narr;
   uint64_t nblocks;       // = first[narr]
-  uint32_t* ticket;       // device: one zeroed counter per digit
+  uint32_t* ticket;       // device: the digit passes' tickets (zeroed)
   uint32_t* lsd;          // device: the digits that some array's LSD passes take (zeroed; set by the plans)
 };
-// stage 0 = histograms, 1 = the pass of `digit`
-cudaError_t launch_radix_batched(const BatchRadix& br, int R, int stage, uint32_t digit, cudaStream_t st);
+// stage 0 = histograms, 1 = the digit passes
+cudaError_t launch_radix_batched(const BatchRadix& br, int R, int stage, cudaStream_t st);
 // Batched hybrid sort (sort_hybrid.cu): every array's plan (digit offsets, its mode: kBatchOnChip, 2 or 0,
 // its ranges in the lists of classes 0..4), the partition of the arrays in mode 2, then one launch per
 // class. The ORP's last pass writes the output buffer in either mode (both count as even).
