@@ -162,7 +162,8 @@ __device__ __forceinline__ unsigned long long st_word(unsigned long long state, 
 // Exclusive prefix of tile `tile` over its predecessors (decoupled look-back, one thread). The
 // word of tile j is status[j * stride]. Spins with a limit; on timeout raises ctrl->timeout and
 // returns the prefix gathered so far. Each step issues the loads of W predecessors at once
-// (independent loads, one round-trip per W tiles), then folds them in order, waiting (bounded) on any not yet published.
+// (independent loads, one round-trip per W tiles), then folds them in order, waiting (bounded) on any
+// not yet published.
 template <int W>
 __device__ __forceinline__ unsigned long long lookback_window(const unsigned long long* status, uint64_t tile,
                                                               uint64_t stride, uint32_t tag, Ctrl* ctrl) {

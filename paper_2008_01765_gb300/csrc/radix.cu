@@ -3,8 +3,7 @@
 // Onesweep organisation: one histogram pass gives the counts of all 8-bit digits at once; each
 // digit then takes one pass that ranks a tile of records stably per digit (one ballot per digit
 // bit + per-warp counters), finds the tile's global offset per digit by decoupled look-back over
-// the tiles in ticket order, stages the tile in shared memory in digit order and writes it out
-// in runs.
+// the tiles in ticket order, puts the records' places in digit order and writes the tile out in runs.
 // A digit on which every key agrees is skipped (the pass would be the identity); the buffers
 // alternate so that the last pass that runs writes the final output.
 #include "common.cuh"
