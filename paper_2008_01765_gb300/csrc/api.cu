@@ -1367,17 +1367,39 @@ bos_status batch_check_in(const BatchIn& b, const BatchLayout& L, void* d_ws, si
   return BOS_OK;
 }
 
-// Writes the descriptors of `sel` (synchronous copy from host memory).
+// Descriptor bytes on the host. A copy from them may read them until the stream has passed it (pageable
+// memory need not be staged: the device can read it directly), so they go only after that.
+struct DescBytes {
+  std::vector<char> bytes;
+  cudaStream_t st = nullptr;
+  bool in_flight = false;  // a copy on st has not been waited for
+  ~DescBytes() {
+    if (in_flight && cudaStreamSynchronize(st) != cudaSuccess) (void)cudaGetLastError();
+  }
+};
+
+// Enqueues the copy of the descriptors of `sel`, which `desc` holds until the stream has passed it.
+bos_status batch_copy(const BatchIn& b, const BatchLayout& L, char* ws, const std::vector<uint32_t>& sel,
+                      const std::vector<uint32_t>& attempt, std::vector<BatchLaunch>* launches,
+                      cudaStream_t st, DescBytes* desc) {
+  size_t used = 0;
+  const bos_status s = batch_build(b, L, ws, sel, attempt, launches, &desc->bytes, &used);
+  if (s != BOS_OK || !used) return s;
+  desc->st = st;
+  desc->in_flight = true;
+  BOS_CUDA(cudaMemcpyAsync(ws + L.desc_off, desc->bytes.data(), used, cudaMemcpyHostToDevice, st));
+  return BOS_OK;
+}
+
+// Writes the descriptors of `sel` (a copy from host memory that has ended when the call returns).
 bos_status batch_prepare(const BatchIn& b, const BatchLayout& L, char* ws, const std::vector<uint32_t>& sel,
                          const std::vector<uint32_t>& attempt, std::vector<BatchLaunch>* launches,
-                         cudaStream_t st, bool wait = true) {
-  std::vector<char> desc;
-  size_t used = 0;
-  bos_status s = batch_build(b, L, ws, sel, attempt, launches, &desc, &used);
+                         cudaStream_t st) {
+  DescBytes desc;
+  const bos_status s = batch_copy(b, L, ws, sel, attempt, launches, st, &desc);
   if (s != BOS_OK) return s;
-  // a copy from pageable memory has left the host buffer when the call returns
-  if (used) BOS_CUDA(cudaMemcpyAsync(ws + L.desc_off, desc.data(), used, cudaMemcpyHostToDevice, st));
-  if (wait) BOS_CUDA(cudaStreamSynchronize(st));
+  BOS_CUDA(cudaStreamSynchronize(st));
+  desc.in_flight = false;
   return BOS_OK;
 }
 
@@ -1592,10 +1614,13 @@ bos_status bos_sort_batched(const void* d_in, void* d_out, const uint64_t* h_off
   if (s != BOS_OK) return s;
   if ((s = batch_check_in(b, L, d_ws, ws_bytes)) != BOS_OK) return s;
   std::vector<BatchLaunch> launches;
-  s = batch_prepare(b, L, (char*)d_ws, all_arrays(num), std::vector<uint32_t>(num, 0), &launches, (cudaStream_t)stream, false);
+  DescBytes desc;  // until batch_collect has synchronised the stream
+  s = batch_copy(b, L, (char*)d_ws, all_arrays(num), std::vector<uint32_t>(num, 0), &launches, (cudaStream_t)stream, &desc);
   if (s != BOS_OK) return s;
   if ((s = batch_enqueue(L, (char*)d_ws, launches, (cudaStream_t)stream)) != BOS_OK) return s;
-  return batch_collect(b, L, (char*)d_ws, (cudaStream_t)stream, h_attempts);
+  s = batch_collect(b, L, (char*)d_ws, (cudaStream_t)stream, h_attempts);
+  if (s != BOS_ERR_CUDA) desc.in_flight = false;  // every other status comes after the synchronisation
+  return s;
 }
 
 bos_status bos_shard_layout(uint64_t n, uint32_t G, const bos_params* p, bos_shard_layout_t* out) {
