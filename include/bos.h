@@ -292,6 +292,10 @@ bos_status bos_trace_attach_digest(void* d_buf, size_t bytes);
 bos_status bos_selftest_philox(const uint32_t* d_ctr, const uint32_t* d_key, uint32_t* d_out,
                                uint32_t* d_out_curand, uint64_t n, void* stream);
 
+/* Self-test hook for the pinned host block that bos_orp / bos_sort share: the slots that no call holds
+ * (0 also while the block does not exist). A call that finds none gives the same result. */
+uint32_t bos_selftest_host_slots(void);
+
 /* Kernel timing for benchmarks (no counterpart in the paper). While enabled, every launch of
  * bos_orp / bos_sort / bos_bitonic_sort is bracketed by CUDA events recorded on the call's
  * stream; each kernel class accumulates its launches, device milliseconds and algorithmic bytes

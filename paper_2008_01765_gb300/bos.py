@@ -124,6 +124,7 @@ def lib():
         L.bos_version.restype = _u32
         L.bos_selftest_philox.argtypes = [_vp, _vp, _vp, _vp, _u64, _vp]
         L.bos_selftest_philox.restype = ctypes.c_int
+        L.bos_selftest_host_slots.restype = _u32
         L.bos_orp_noalloc.argtypes = [_vp, _vp, _u64, ctypes.POINTER(Params), _vp,
                                       ctypes.POINTER(Info)]
         L.bos_orp_noalloc.restype = ctypes.c_int

@@ -1930,6 +1930,11 @@ const char* bos_status_str(bos_status s) {
 
 uint32_t bos_version(void) { return (0u << 16) | 1u; }
 
+uint32_t bos_selftest_host_slots(void) {
+  std::lock_guard<std::mutex> g(g_slots.mu);
+  return g_slots.base ? (uint32_t)(kHostSlots - __builtin_popcount(g_slots.busy)) : 0u;
+}
+
 bos_status bos_profile_enable(int on) {
   std::lock_guard<std::mutex> g(g_state_mu);
   if (on && !g_prof.created) {

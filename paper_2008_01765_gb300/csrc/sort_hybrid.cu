@@ -1451,8 +1451,9 @@ cudaError_t launch_r(const HybridArgs& a, int stage, const uint32_t* list, cudaS
     }
     default: {
       if (list[0]) {
-        const uint32_t need = (list[0] + kSThreads / 32 - 1) / (kSThreads / 32);
-        local_small_kernel<R><<<need < (uint32_t)sms * 8 ? need : (unsigned)sms * 8, kSThreads, 0, st>>>(a);
+        // rounded up without a sum: the count is all ones when the host does not know it
+        const uint32_t need = (list[0] - 1) / (kSThreads / 32) + 1, most = (uint32_t)sms * 8;
+        local_small_kernel<R><<<need < most ? need : most, kSThreads, 0, st>>>(a);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
       }
       if ((e = launch_bins<R, 1>(a, list[1], sms, st)) != cudaSuccess) return e;

@@ -1,4 +1,12 @@
-"""Host memory that the GPU reads or writes while a call runs: it outlives the work that uses it."""
+"""Host memory that the GPU reads or writes while a call runs: it outlives the work that uses it, and calls
+that find no slot of the shared pinned block are as good as those that do. What depends on the state of a
+whole process runs in a child (this file with the function's name)."""
+import os
+import subprocess
+import sys
+import threading
+import time
+
 import numpy as np
 import pytest
 
@@ -6,6 +14,9 @@ import oracle
 from paper_2008_01765_gb300 import inputs
 
 pytestmark = pytest.mark.gpu
+
+
+SLOTS = 12
 
 
 @pytest.fixture(scope="module")
@@ -18,6 +29,20 @@ def bos():
     from paper_2008_01765_gb300 import bos as b
     b.lib()
     return b
+
+
+def _child(name, **env):
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    r = subprocess.run([sys.executable, "-m", "tests.test_gpu_host_state", name], cwd=root, env={**os.environ, **env},
+                       capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0, r.stdout + r.stderr
+
+
+def _keys(n, rec_bytes, shape):
+    recs = inputs.make_records(n, rec_bytes, "uniform", seed=n)
+    if shape == "two":  # crowds one value of the top digit from kCap on: LSD passes
+        recs["key"] = recs["key"] & recs["key"].dtype.type(1 << 7)
+    return recs
 
 
 def test_batch_descriptors_outlive_their_copy(bos):
@@ -45,3 +70,67 @@ def test_batch_descriptors_outlive_their_copy(bos):
             lo, hi = int(offs[j]), int(offs[j + 1])
             ref, _ = (oracle.sort if ops[j] else oracle.orp)(recs[lo:hi], 512, int(seeds[j]), method=oracle.CLOSED)
             np.testing.assert_array_equal(got[lo:hi], ref, err_msg=f"array {j}")
+
+
+# every mode of the sort: on chip (classes 0 to 5), one partition, two partitions, LSD passes, one key
+NO_SLOT_CASES = [(1, 16, "uniform"), (200, 8, "uniform"), (1000, 16, "uniform"), (2000, 8, "two"), (4096, 16, "uniform"),
+                 (9000, 16, "two"), (19000, 16, "uniform"), (19000, 16, "two"), (28000, 8, "uniform"),
+                 (70001, 16, "uniform"), (1 << 20, 8, "uniform"), (1 << 20, 16, "two"), ((1 << 23) + 1, 16, "uniform")]
+
+
+def child_no_slot():
+    import torch
+    from paper_2008_01765_gb300 import bos
+    jobs = []
+    for n, rec, shape in NO_SLOT_CASES:
+        recs = _keys(n, rec, shape)
+        x = bos.to_device(recs)
+        p = bos.params(rec, 512, 5)
+        jobs.append((recs, rec, x, torch.empty_like(x), bos.alloc_workspace(bos.workspace_bytes(n, p))))
+    for rec in (8, 16):  # every kernel of the sort once: loading one late may wait for the sleeping calls
+        for n, shape in [(200, "uniform"), (1000, "uniform"), (2000, "uniform"), (4096, "uniform"), (9000, "uniform"),
+                         (14000, "two"), (19000, "two"), (28000, "two"), (70001, "uniform"), (1 << 20, "two"),
+                         (1 << 24, "uniform")]:
+            bos.sort(bos.to_device(_keys(n, rec, shape)), rec, Z=512, seed=5)
+    small = bos.to_device(_keys(64, 16, "uniform"))
+    held = [(torch.cuda.Stream(), torch.empty_like(small), bos.alloc_workspace(1 << 20)) for _ in range(SLOTS)]
+    main = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    free = bos.lib().bos_selftest_host_slots
+
+    def hold(stream, out, ws):  # a call that waits for its stream holds its slot meanwhile
+        with torch.cuda.stream(stream):
+            torch.cuda._sleep(1_000_000_000)  # about half a second
+        bos.orp(small, 16, Z=512, seed=1, out=out, workspace=ws, stream=stream)
+
+    assert free() == SLOTS
+    threads = [threading.Thread(target=hold, args=h) for h in held]
+    for t in threads:
+        t.start()
+    end = time.time() + 0.3
+    while free() and time.time() < end:
+        time.sleep(0.001)
+    assert free() == 0
+    infos = []
+    for recs, rec, x, out, ws in jobs:
+        infos.append(bos.sort(x, rec, Z=512, seed=5, out=out, workspace=ws, stream=main)[1])
+        assert free() == 0, f"{len(recs)} x {rec}: the slots were not held long enough"
+    for t in threads:
+        t.join()
+    assert free() == SLOTS
+    modes = set()
+    for (recs, rec, x, out, ws), info in zip(jobs, infos):
+        ref, rinfo = oracle.sort(recs, 512, 5, method=oracle.CLOSED)
+        assert info.attempts == rinfo.attempts
+        modes.add(info.sort_mode)
+        np.testing.assert_array_equal(bos.to_host(out, recs.dtype), ref, err_msg=f"{len(recs)} x {rec}")
+    assert modes == {0, 1, 2, 3}
+
+
+def test_sort_without_a_host_slot(bos):
+    # twelve calls hold the twelve slots; a queue per stream, so that the others run meanwhile
+    _child("child_no_slot", CUDA_DEVICE_MAX_CONNECTIONS="32")
+
+
+if __name__ == "__main__":
+    globals()[sys.argv[1]]()
