@@ -20,7 +20,7 @@
  *   - Every pointer named d_* is a device pointer owned by the caller. No call allocates or
  *     frees device memory, prints or aborts; errors are reported by status (host-side scratch of
  *     the batched calls is ordinary heap memory, and bos_orp / bos_sort share one 4 KiB block of
- *     pinned host memory, allocated on the first call). The library image itself holds one fixed
+ *     pinned host memory, allocated by the first of these calls). The library image itself holds one fixed
  *     device array, the BOS_NOALLOC_SCRATCH_BYTES scratch of bos_orp_noalloc, on every GPU
  *     where its kernels are loaded.
  *   - `stream` is a cudaStream_t (NULL = the legacy default stream). Work is stream-ordered.
@@ -140,7 +140,8 @@ bos_status bos_orp(const void* d_in, void* d_out, uint64_t n, const bos_params* 
  *     workspace for n fits; otherwise the call returns BOS_ERR_WORKSPACE and touches nothing.
  *     (bos_workspace_bytes(n, p) <= BOS_NOALLOC_SCRATCH_BYTES is a sufficient check; with
  *     Z = 512 every n <= 2^19 fits for 16-byte records and every n <= 2^20 for 8-byte records.)
- *   - no allocation: the call makes no cudaMalloc / cudaFree or other allocating call. Every call
+ *   - no allocation: the call makes no cudaMalloc / cudaFree or other allocating call (the pinned host
+ *     block of bos_orp / bos_sort it uses only where it exists already). Every call
  *     looks up the scratch's device address on the current device (cudaGetSymbolAddress); on the
  *     first call on a device that lookup also loads the library's kernels there.
  *   - synchronisation: like bos_orp, the call synchronises `stream` after every attempt to read

@@ -133,7 +133,8 @@ struct Zeroer {
 
 // Host words of the calls in flight: the sort's plan and the control block's copy, in pinned mapped
 // memory (a copy to pageable memory takes 5 us longer, and the plan can be read while the ORP runs).
-// kHostSlots slots, allocated once (4 KiB); a call that finds none free works without.
+// kHostSlots slots, allocated once (4 KiB) by a call that may allocate; a call that finds none free, or no
+// block where it may not allocate one, works without.
 struct HostSlot {
   HostPlan plan;
   uint32_t pad[7];
@@ -152,9 +153,9 @@ struct SlotLease {
   uint32_t seq = 0;
   int i = -1;
   bool clean = false;  // the stream has been synchronised: nothing writes the slot any more
-  SlotLease() {
+  explicit SlotLease(bool may_alloc) {
     std::lock_guard<std::mutex> g(g_slots.mu);
-    if (!g_slots.tried) {
+    if (!g_slots.tried && may_alloc) {
       g_slots.tried = true;
       void* p = nullptr;
       if (cudaHostAlloc(&p, kHostSlots * sizeof(HostSlot), cudaHostAllocPortable | cudaHostAllocMapped) == cudaSuccess)
@@ -640,8 +641,9 @@ bool overlaps(const void* a, size_t na, const void* b, size_t nb) {
     }                                    \
   } while (0)
 
+// may_alloc: the call may allocate host memory (the pinned slots).
 bos_status run(const void* d_in, void* d_out, uint64_t n, const bos_params* p, void* d_ws,
-               size_t ws_bytes, void* stream, bos_info* info, bool sort) {
+               size_t ws_bytes, void* stream, bos_info* info, bool sort, bool may_alloc = true) {
   Plan pl;
   const bool plan_only = p && (p->flags & BOS_FLAG_PLAN_ONLY);
   bos_status s = (n && !plan_only) ? device_plan(n, p, sort, &pl) : make_plan(n, p, sort, &pl);
@@ -745,7 +747,7 @@ bos_status run(const void* d_in, void* d_out, uint64_t n, const bos_params* p, v
     ha.ctrl = ctrl;
   }
 
-  SlotLease slot;
+  SlotLease slot(may_alloc);
   for (uint32_t attempt = 0; attempt < max_attempts; ++attempt) {
     slot.clean = false;
     Zeroer zero;
@@ -1526,7 +1528,7 @@ size_t orp_workspace_bytes(uint64_t n, const bos_params* p) {
 
 bos_status orp_with_workspace(const void* d_in, void* d_out, uint64_t n, const bos_params* p,
                               void* d_ws, size_t ws_bytes, void* stream, bos_info* info) {
-  return run(d_in, d_out, n, p, d_ws, ws_bytes, stream, info, false);
+  return run(d_in, d_out, n, p, d_ws, ws_bytes, stream, info, false, false);
 }
 
 }  // namespace bos

@@ -132,5 +132,25 @@ def test_sort_without_a_host_slot(bos):
     _child("child_no_slot", CUDA_DEVICE_MAX_CONNECTIONS="32")
 
 
+def child_noalloc_first():
+    from paper_2008_01765_gb300 import bos
+    recs = _keys(5000, 16, "uniform")
+    x = bos.to_device(recs)
+    ref, _ = oracle.orp(recs, 512, 3, method=oracle.CLOSED)
+    free = bos.lib().bos_selftest_host_slots
+    for block in (0, SLOTS):  # before the block exists, and after bos_orp has made it
+        for _ in range(2):
+            out, _ = bos.orp_noalloc(x, 16, Z=512, seed=3)
+            np.testing.assert_array_equal(bos.to_host(out, recs.dtype), ref)
+            assert free() == block
+        bos.orp(x, 16, Z=512, seed=3)
+        assert free() == SLOTS
+
+
+def test_noalloc_allocates_no_host_block(bos):
+    # the process's first call is bos_orp_noalloc: the pinned block must not come into being
+    _child("child_noalloc_first")
+
+
 if __name__ == "__main__":
     globals()[sys.argv[1]]()
