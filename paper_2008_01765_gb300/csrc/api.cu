@@ -152,8 +152,9 @@ struct SlotLease {
   HostSlot* h = nullptr;
   uint32_t seq = 0;
   int i = -1;
+  cudaStream_t st;
   bool clean = false;  // the stream has been synchronised: nothing writes the slot any more
-  explicit SlotLease(bool may_alloc) {
+  SlotLease(cudaStream_t s, bool may_alloc) : st(s) {
     std::lock_guard<std::mutex> g(g_slots.mu);
     if (!g_slots.tried && may_alloc) {
       g_slots.tried = true;
@@ -175,9 +176,19 @@ struct SlotLease {
       }
   }
   ~SlotLease() {
-    if (i < 0 || !clean) return;  // a call that failed halfway may still have its plan kernel in flight
+    if (i < 0 || !(clean || idle())) return;
     std::lock_guard<std::mutex> g(g_slots.mu);
     g_slots.busy &= ~(1u << i);
+  }
+  // After a call that failed halfway: waits for its plan kernel and its copy, which write the slot. They never
+  // run if they went to a capture, which the failure has invalidated. Otherwise the context is lost, and
+  // the slot with it.
+  bool idle() const {
+    if (cudaStreamSynchronize(st) == cudaSuccess) return true;
+    (void)cudaGetLastError();
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(st, &cs) != cudaSuccess) (void)cudaGetLastError();
+    return cs == cudaStreamCaptureStatusInvalidated;
   }
   // The next attempt's plan gets a number of its own (the stream has been synchronised).
   void renew() {
@@ -187,7 +198,7 @@ struct SlotLease {
     seq = ++g_slots.seq ? g_slots.seq : ++g_slots.seq;
   }
   // Waits until the plan kernel has published; false if the stream ended or failed without it.
-  bool wait(cudaStream_t st) const {
+  bool wait() const {
     for (uint32_t spin = 1;; ++spin) {
       if (__atomic_load_n(&h->plan.seq, __ATOMIC_ACQUIRE) == seq) return true;
       if ((spin & 0xFFFu) == 0) {
@@ -747,7 +758,7 @@ bos_status run(const void* d_in, void* d_out, uint64_t n, const bos_params* p, v
     ha.ctrl = ctrl;
   }
 
-  SlotLease slot(may_alloc);
+  SlotLease slot(st, may_alloc);
   for (uint32_t attempt = 0; attempt < max_attempts; ++attempt) {
     slot.clean = false;
     Zeroer zero;
@@ -876,7 +887,7 @@ bos_status run(const void* d_in, void* d_out, uint64_t n, const bos_params* p, v
       uint32_t mode = 4, live = 0xFFFFFFFFu, list[kSortClasses];
       for (uint32_t& c : list) c = 0xFFFFFFFFu;
       if (hybrid && slot.h) {
-        if (!slot.wait(st)) return BOS_ERR_CUDA;
+        if (!slot.wait()) return BOS_ERR_CUDA;
         mode = slot.h->plan.mode;
         live = slot.h->plan.live;
         for (uint32_t c = 0; c < kSortClasses; ++c) list[c] = slot.h->plan.list[c];

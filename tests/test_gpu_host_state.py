@@ -1,6 +1,7 @@
 """Host memory that the GPU reads or writes while a call runs: it outlives the work that uses it, and calls
 that find no slot of the shared pinned block are as good as those that do. What depends on the state of a
 whole process runs in a child (this file with the function's name)."""
+import ctypes
 import os
 import subprocess
 import sys
@@ -150,6 +151,34 @@ def child_noalloc_first():
 def test_noalloc_allocates_no_host_block(bos):
     # the process's first call is bos_orp_noalloc: the pinned block must not come into being
     _child("child_noalloc_first")
+
+
+def child_failed_calls():
+    import torch
+    from paper_2008_01765_gb300 import bos
+    recs = _keys(5000, 16, "uniform")
+    x = bos.to_device(recs)
+    out, ws = torch.empty_like(x), bos.alloc_workspace(1 << 24)
+    ref, _ = oracle.sort(recs, 512, 3, method=oracle.CLOSED)
+    bos.sort(x, 16, Z=512, seed=3, out=out, workspace=ws)
+    bos.orp(x, 16, Z=512, seed=3, out=out, workspace=ws)
+    stream = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    rt = ctypes.CDLL("libcudart.so.13")
+    handle, graph = ctypes.c_void_p(stream.cuda_stream), ctypes.c_void_p()
+    for j in range(2 * SLOTS):  # a call that synchronises cannot be captured: it fails halfway
+        assert rt.cudaStreamBeginCapture(handle, 2) == 0  # 2: relaxed
+        with pytest.raises(bos.BosError):
+            (bos.sort if j % 2 else bos.orp)(x, 16, Z=512, seed=3, out=out, workspace=ws, stream=stream)
+        assert rt.cudaStreamEndCapture(handle, ctypes.byref(graph)) != 0  # invalidated
+        rt.cudaGetLastError()
+        assert bos.lib().bos_selftest_host_slots() == SLOTS, j
+    bos.sort(x, 16, Z=512, seed=3, out=out, workspace=ws, stream=stream)
+    np.testing.assert_array_equal(bos.to_host(out, recs.dtype), ref)
+
+
+def test_failed_calls_give_their_slots_back(bos):
+    _child("child_failed_calls")
 
 
 if __name__ == "__main__":
