@@ -20,7 +20,8 @@
  *   - Every pointer named d_* is a device pointer owned by the caller. No call allocates or
  *     frees device memory, prints or aborts; errors are reported by status (host-side scratch of
  *     the batched calls is ordinary heap memory, and bos_orp / bos_sort share one 4 KiB block of
- *     pinned host memory, allocated by the first of these calls). The library image itself holds one fixed
+ *     pinned host memory, allocated by the first of these calls and anew after a
+ *     device reset, which must not run while one of them does). The library image itself holds one fixed
  *     device array, the BOS_NOALLOC_SCRATCH_BYTES scratch of bos_orp_noalloc, on every GPU
  *     where its kernels are loaded.
  *   - `stream` is a cudaStream_t (NULL = the legacy default stream). Work is stream-ordered.

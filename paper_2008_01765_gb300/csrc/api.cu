@@ -7,6 +7,8 @@
 #include <utility>
 #include <vector>
 
+#include <cuda.h>  // types only: the driver's function is looked up at run time
+
 #include "bos.h"
 #include "internal.h"
 
@@ -144,31 +146,68 @@ constexpr int kHostSlots = 12;
 struct HostSlots {
   std::mutex mu;
   HostSlot* base = nullptr;
-  bool tried = false;
+  unsigned long long id = 0;  // the allocation's id, which no later allocation gets
+  uint32_t gen = 0;           // counts the allocations
   uint32_t busy = 0, seq = 0;
 };
 HostSlots g_slots;
+
+using PointerQuery = CUresult (*)(void*, CUpointer_attribute, CUdeviceptr);
+PointerQuery pointer_query() {
+  static const PointerQuery f = [] {
+    void* p = nullptr;
+    cudaDriverEntryPointQueryResult r = cudaDriverEntryPointSymbolNotFound;
+    if (cudaGetDriverEntryPointByVersion("cuPointerGetAttribute", &p, 12000, cudaEnableDefault, &r) != cudaSuccess)
+      (void)cudaGetLastError();
+    return r == cudaDriverEntryPointSuccess ? (PointerQuery)p : nullptr;
+  }();
+  return f;
+}
+
+// The id of the live allocation that holds p. A device reset (or the end of the context that made it) frees
+// the block under the library, and its address is given out again: the same address came back in three of
+// three tries, with another id. Both queries together take 0.09 us; the runtime's, first, also binds the
+// thread to a context.
+bool allocation_id(const void* p, unsigned long long* id) {
+  cudaPointerAttributes a{};
+  if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+    (void)cudaGetLastError();
+    return false;
+  }
+  return a.type == cudaMemoryTypeHost &&
+         pointer_query()(id, CU_POINTER_ATTRIBUTE_BUFFER_ID, (CUdeviceptr)p) == CUDA_SUCCESS;
+}
+
 struct SlotLease {
   HostSlot* h = nullptr;
-  uint32_t seq = 0;
+  uint32_t seq = 0, gen = 0;
   int i = -1;
   cudaStream_t st;
   bool clean = false;  // the stream has been synchronised: nothing writes the slot any more
   SlotLease(cudaStream_t s, bool may_alloc) : st(s) {
     std::lock_guard<std::mutex> g(g_slots.mu);
-    if (!g_slots.tried && may_alloc) {
-      g_slots.tried = true;
+    unsigned long long id = 0;
+    if (g_slots.base && !(allocation_id(g_slots.base, &id) && id == g_slots.id)) {  // gone with its context
+      g_slots.base = nullptr;
+      g_slots.busy = 0;
+    }
+    if (!g_slots.base && may_alloc && pointer_query()) {
       void* p = nullptr;
-      if (cudaHostAlloc(&p, kHostSlots * sizeof(HostSlot), cudaHostAllocPortable | cudaHostAllocMapped) == cudaSuccess)
-        g_slots.base = (HostSlot*)p;
-      else
+      if (cudaHostAlloc(&p, kHostSlots * sizeof(HostSlot), cudaHostAllocPortable | cudaHostAllocMapped) != cudaSuccess)
         (void)cudaGetLastError();
+      else if (allocation_id(p, &g_slots.id)) {
+        g_slots.base = (HostSlot*)p;
+        ++g_slots.gen;
+      } else {
+        (void)cudaFreeHost(p);
+      }
     }
     if (!g_slots.base) return;
     for (int x = 0; x < kHostSlots; ++x)
       if (!((g_slots.busy >> x) & 1u)) {
         g_slots.busy |= 1u << x;
         i = x;
+        gen = g_slots.gen;
         h = g_slots.base + x;
         seq = ++g_slots.seq ? g_slots.seq : ++g_slots.seq;
         h->plan.seq = 0;
@@ -178,7 +217,7 @@ struct SlotLease {
   ~SlotLease() {
     if (i < 0 || !(clean || idle())) return;
     std::lock_guard<std::mutex> g(g_slots.mu);
-    g_slots.busy &= ~(1u << i);
+    if (gen == g_slots.gen) g_slots.busy &= ~(1u << i);
   }
   // After a call that failed halfway: waits for its plan kernel and its copy, which write the slot. They never
   // run if they went to a capture, which the failure has invalidated. Otherwise the context is lost, and

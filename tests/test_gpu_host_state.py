@@ -181,5 +181,54 @@ def test_failed_calls_give_their_slots_back(bos):
     _child("child_failed_calls")
 
 
+def child_reset():
+    # no torch here: its allocator would not survive the reset
+    from paper_2008_01765_gb300 import bos
+    rt = ctypes.CDLL("libcudart.so.13")
+    rt.cudaMalloc.argtypes = [ctypes.POINTER(ctypes.c_void_p), ctypes.c_size_t]
+    rt.cudaHostAlloc.argtypes = [ctypes.POINTER(ctypes.c_void_p), ctypes.c_size_t, ctypes.c_uint]
+    rt.cudaMemcpy.argtypes = [ctypes.c_void_p, ctypes.c_void_p, ctypes.c_size_t, ctypes.c_int]
+    L, n = bos.lib(), 5000
+    recs = _keys(n, 16, "uniform")
+    p = bos.params(16, 512, 3)
+    need = bos.workspace_bytes(n, p)
+    ref = {"bos_sort": oracle.sort(recs, 512, 3, method=oracle.CLOSED)[0]}
+    ref["bos_orp"] = ref["bos_orp_noalloc"] = oracle.orp(recs, 512, 3, method=oracle.CLOSED)[0]
+
+    def alloc(nbytes):
+        q = ctypes.c_void_p()
+        assert rt.cudaMalloc(ctypes.byref(q), nbytes) == 0
+        return q
+
+    def call(name):
+        x, out, ws = alloc(n * 16), alloc(n * 16), alloc(need)
+        assert rt.cudaMemcpy(x, recs.ctypes.data, n * 16, 1) == 0
+        args = (x, out, n, ctypes.byref(p)) + ((None, None) if name == "bos_orp_noalloc" else (ws, need, None, None))
+        assert getattr(L, name)(*args) == bos.OK, name
+        got = np.zeros_like(recs)
+        assert rt.cudaMemcpy(got.ctypes.data, out, n * 16, 2) == 0
+        np.testing.assert_array_equal(got, ref[name], err_msg=name)
+
+    for order in (("bos_sort", "bos_orp"), ("bos_orp", "bos_sort"), ("bos_orp_noalloc", "bos_sort")):
+        call("bos_sort")
+        assert L.bos_selftest_host_slots() == SLOTS
+        assert rt.cudaDeviceReset() == 0
+        mine = []  # pinned memory of the caller's, some of it where the library's block was
+        for _ in range(8):
+            q = ctypes.c_void_p()
+            assert rt.cudaHostAlloc(ctypes.byref(q), 4096, 3) == 0  # portable, mapped
+            ctypes.memset(q, 0x5A, 4096)
+            mine.append(q)
+        for name in order:
+            call(name)
+        assert L.bos_selftest_host_slots() == SLOTS
+        assert all(ctypes.string_at(q, 4096) == b"\x5a" * 4096 for q in mine)
+
+
+def test_host_block_after_a_device_reset(bos):
+    # the reset ends the process's own context, and the pinned block with it
+    _child("child_reset")
+
+
 if __name__ == "__main__":
     globals()[sys.argv[1]]()
