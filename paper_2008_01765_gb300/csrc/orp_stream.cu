@@ -71,6 +71,8 @@ constexpr uint32_t kListWords = 4096;   // list places of all output buckets tog
                                         // 0x8000 | slot index, or 0xFFFF when unused
 constexpr uint32_t kBatchSlots = 2048;  // most slots per batch of a middle pass (four per thread)
 constexpr uint32_t kBatchRecs = 1024;   // most records per batch of the first pass (two per thread)
+constexpr uint32_t kWhole = 2 * kBatchSlots;  // round size of a batch's first round: all of it, and above every
+                                              // size of a redone round (doubled only while below the batch's)
 constexpr uint32_t kSub = 16;           // slots per round when a batch is redone
 constexpr uint32_t kDone = (kBatchSlots + 256 * 7) / 8;  // most chunks a batch completes
 constexpr uint32_t kAcc = 11;           // level counters per lane of the last warp
@@ -325,7 +327,7 @@ __device__ __forceinline__ void orp_stream_body(const PassArgs& a, const StreamL
   uint64_t q = q0;
   uint32_t g = 0, s = 0, st = 0, par = 0;  // batch g is batch s of subproblem q; its stage and the stage's parity
   uint32_t pb = 0;      // the round's buffer of lists, counts and fills
-  uint32_t rlo = 0, sz = kBatchSlots;  // the round's first slot and size
+  uint32_t rlo = 0, sz = kWhole;  // the round's first slot and size
   bool pend = false;    // the previous round (buffer pb ^ 1) has not been drained yet
   Rec* orec = reinterpret_cast<Rec*>(a.out_rec) + q * D * Z;  // the subproblem's output buckets
   uint32_t* otag = a.out_tag + q * D * Z;
@@ -429,7 +431,7 @@ __device__ __forceinline__ void orp_stream_body(const PassArgs& a, const StreamL
           else
             full = true;
         }
-    } else if (g >= NB && sz == kBatchSlots) {  // once per batch
+    } else if (g >= NB && sz == kWhole) {  // once per batch: a redone round never has this size
       write_tail(q - qstep, s, false);
     }
     if (__syncthreads_or(full)) {
@@ -520,7 +522,7 @@ __device__ __forceinline__ void orp_stream_body(const PassArgs& a, const StreamL
     ++g;
     ++s;
     rlo = 0;
-    sz = kBatchSlots;
+    sz = kWhole;
     if (++st == nst) {
       st = 0;
       par ^= 1u;
