@@ -3,6 +3,9 @@ run in parts, middle passes of a batch."""
 import numpy as np
 import pytest
 
+import oracle
+from paper_2008_01765_gb300 import inputs
+
 pytestmark = pytest.mark.gpu
 
 
@@ -43,3 +46,51 @@ def test_redone_batches_write_every_chunk_once(bos):
         with np.errstate(over="ignore"):
             digests.append((int(s[:, 0].sum()), int(s[:, 1].sum())))
     assert digests[0] == digests[1]
+
+
+def _batch(bos, parts, rec_bytes, Zs, seeds):
+    """Every array as ORP and as sort in one batch, each against the oracle alone."""
+    import torch
+    recs = np.concatenate(parts + parts)
+    sizes = [len(p) for p in parts] * 2
+    offs = np.zeros(len(sizes) + 1, dtype=np.uint64)
+    np.cumsum(sizes, out=offs[1:])
+    ops = np.repeat(np.array([0, 1], dtype=np.uint8), len(parts))
+    x = bos.to_device(recs)
+    b = bos.Batch(x, torch.zeros_like(x), offs, np.array(seeds * 2, dtype=np.uint64), ops, bos.params(rec_bytes, 512, 0),
+                  Zs=np.array(Zs * 2, dtype=np.uint32))
+    att = b.run()
+    got = bos.to_host(b.out, recs.dtype)
+    for j in range(len(sizes)):
+        lo, hi = int(offs[j]), int(offs[j + 1])
+        ref, rinfo = (oracle.sort if ops[j] else oracle.orp)(recs[lo:hi], (Zs * 2)[j], (seeds * 2)[j], method=oracle.CLOSED)
+        assert att[j] == rinfo.attempts, j
+        np.testing.assert_array_equal(got[lo:hi], ref, err_msg=f"array {j}")
+
+
+@pytest.mark.parametrize("rec_bytes", [8, 16])
+def test_batched_middle_passes(bos, rec_bytes):
+    # a batch's streaming plan has 8 levels in its first pass and 4 in the last: a middle pass from L = 13 on;
+    # batches of one, two and four buckets, beside arrays of two passes
+    shapes = [(300000, 128), (5000, 512), ((1 << 20) + 3, 256), ((1 << 21) + 7, 512), (1 << 20, 512)]
+    if rec_bytes == 8:
+        shapes.append(((1 << 23) + 5, 1536))
+    assert [bos.plan(n, rec_bytes, Z).L >= 13 for n, Z in shapes[:5]] == [True, False, True, True, False]
+    parts = [inputs.make_records(n, rec_bytes, "uniform", seed=n) for n, _ in shapes]
+    _batch(bos, parts, rec_bytes, [Z for _, Z in shapes], list(range(31, 31 + len(shapes))))
+
+
+@pytest.mark.parametrize("seed", [52, 293])
+def test_tile_pass_in_parts(bos, seed):
+    # 512 full buckets of Z = 896: five levels in the streaming pass, four in the tile, which has room for 7408
+    # 16-byte records; with these seeds a subproblem holds more and runs in parts
+    n, Z = 256 * 896, 896
+    info = bos.plan(n, 16, Z, k=5, sort=False)
+    assert (info.L, info.passes, info.stream_passes, info.max_k, info.max_cluster) == (9, 2, 1, 5, 1)
+    assert np.bincount(oracle.labels(n, seed, 0, 9) >> 4).max() > 7408
+    recs = inputs.make_records(n, 16, "uniform", seed=seed)
+    ref, rinfo = oracle.orp(recs, Z, seed, method=oracle.CLOSED)
+    out, info = bos.orp(bos.to_device(recs), 16, Z=Z, seed=seed, k=5)
+    assert info.attempts == rinfo.attempts == 1
+    np.testing.assert_array_equal(bos.to_host(out, recs.dtype), ref)
+    _batch(bos, [recs, recs[:70001]], 16, [Z, Z], [seed, 5])
