@@ -1011,8 +1011,8 @@ struct BatchLayout {
 };
 
 // The streaming plan of a batch's array of L levels: one first pass of up to 8 levels (two streaming passes
-// beyond 12 levels) and up to 4 in the last. A batch has subproblems enough for every SM, so the fewest
-// passes are the cheapest. np = 0: the one-CTA-per-subproblem passes (few levels, other bucket sizes).
+// beyond 12 levels) and up to 4 in the last, the fewest passes. np = 0: the one-CTA-per-subproblem passes (few
+// levels, other bucket sizes; or the whole batch, see batch_streams).
 struct BatchStreamZ {  // what the kernels take of one bucket size
   uint32_t Z = 0, kt = 0;
 };
@@ -1034,6 +1034,51 @@ void batch_stream_plan(const bos_params& p, uint32_t L, BatchStreamZ* z, BatchAr
   if (a->np == 3) a->k[1] = S / 2;
   a->k[a->np - 1] = l;
   for (uint32_t x = 1; x < a->np; ++x) a->lvl[x] = a->lvl[x - 1] + a->k[x - 1];
+}
+
+// Whether the arrays with a streaming plan take it, or all of them the one-CTA-per-subproblem passes: the lower
+// of two estimates in microseconds. A launch takes its latency and the rounds of CTAs that the SMs need. The
+// streaming passes move a record at half the cost but have few, long subproblems (16 of up to 160 us for an
+// array of at most 12 levels), so few arrays leave SMs idle, and two more launches; few levels and small buckets
+// give their barriers little to do. Measured both ways in batches of 1 to 2048 arrays of 2^10 to 2^24 records,
+// Z = 32 to 2048 (16-byte ORPs, us, streaming and the other; * the estimate's choice). Z = 512: one array of 2^20
+// 266 and *178, two of 2^20 *306 and 364, 512 of 2^13 693 and *543, 512 of 2^16 *2090 and 3278; Z = 64, 16 of 2^16
+// 303 and *200. The constants are fitted to these 1676 batches: the choice costs 0.4 % over the better route on
+// average, at most 11 % where it streams and 20 % where it does not.
+bool batch_streams(const std::vector<BatchArr>& arr, int R) {
+  struct Launch {
+    double us = 0, most = 0;
+    uint64_t units = 0;
+    void add(double u, uint64_t n) {
+      us += u * (double)n;
+      units += n;
+      most = u > most ? u : most;
+    }
+    double time() const {
+      const double sms = kPlanSms;
+      if (!units) return 0;
+      const double t = units < 4 * kPlanSms ? us / (double)units * (double)((units + kPlanSms - 1) / kPlanSms) : us / sms;
+      return t > most ? t : most;
+    }
+  };
+  Launch stream[2], last;
+  double kslots = 0, generic = 0;  // kslots: 1024 slots
+  uint32_t max_Z = 0, npass = 0;
+  for (const BatchArr& a : arr) {
+    if (!a.np) continue;
+    const uint32_t Z = a.pl.Z, l = a.k[a.np - 1];
+    const double ks = (double)a.pl.B * Z / 1024.0, fill = (double)a.pl.n / ((double)a.pl.B * Z);
+    for (uint32_t x = 0; x + 1 < a.np; ++x) stream[x].add(orp_stream_sub_us(Z, a.k[x], x == 0, fill), a.pl.B >> a.k[x]);
+    last.add(orp_last_sub_us(R, Z, l, fill) + 2.7, a.pl.B >> l);
+    kslots += ks;
+    generic += a.pl.npass * ks;
+    npass = a.pl.npass > npass ? a.pl.npass : npass;
+    max_Z = Z > max_Z ? Z : max_Z;
+  }
+  double t_stream = 48.0 + 0.05 * max_Z + 1.05 * kslots / kPlanSms + last.time();  // loads, table, last pass
+  for (const Launch& s : stream)
+    if (s.units) t_stream += 11.0 + s.time();
+  return t_stream < 13.0 + 0.03 * max_Z + 9.0 * npass + (R == 8 ? 3.6 : 4.1) * generic / kPlanSms;
 }
 
 bos_status batch_layout(const BatchIn& b, BatchLayout* L) {
@@ -1109,6 +1154,9 @@ bos_status batch_layout(const BatchIn& b, BatchLayout* L) {
   L->list_off = off;
   off = align256(off + (size_t)(kSortClasses - 1) * L->list_cap * sizeof(uint4));
   L->total = off;
+  // (the workspace holds either route, so it does not shrink where a batch grows)
+  if (!batch_streams(L->arr, L->R))
+    for (BatchArr& a : L->arr) a.np = 0;
   return BOS_OK;
 }
 

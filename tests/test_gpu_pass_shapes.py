@@ -94,3 +94,34 @@ def test_tile_pass_in_parts(bos, seed):
     assert info.attempts == rinfo.attempts == 1
     np.testing.assert_array_equal(bos.to_host(out, recs.dtype), ref)
     _batch(bos, [recs, recs[:70001]], 16, [Z, Z], [seed, 5])
+
+
+@pytest.mark.parametrize("rec_bytes", [8, 16])
+@pytest.mark.parametrize("count,n,Z,streams", [(1, 1 << 20, 512, False), (48, 1 << 17, 512, True), (64, 1 << 16, 64, False),
+                                               (256, 1 << 12, 256, False), (2, (1 << 20) + 5, 1024, True)])
+def test_batch_route(bos, rec_bytes, count, n, Z, streams):
+    # streaming passes only where the batch has subproblems enough for them and buckets long enough (elsewhere
+    # they took up to 4 times as long); the digest of the accesses tells the routes apart, the results agree
+    import torch
+    recs = inputs.make_records(count * n, rec_bytes, "uniform", seed=count)
+    offs = np.arange(count + 1, dtype=np.uint64) * np.uint64(n)
+    ops = np.zeros(count, dtype=np.uint8)
+    seeds = np.arange(7, 7 + count, dtype=np.uint64)
+    x = bos.to_device(recs)
+    got, digest = [], []
+    for flags in (0, bos.FLAG_NO_STREAM):
+        b = bos.Batch(x, torch.zeros_like(x), offs, seeds, ops, bos.params(rec_bytes, Z, 0, flags=flags))
+        buf = torch.zeros(512, dtype=torch.int64, device="cuda")
+        bos.trace_attach_digest(buf)
+        try:
+            att = b.run()
+        finally:
+            bos.trace_attach_digest(None)
+        assert att.max() == 1
+        digest.append(buf.cpu().numpy().view(np.uint64).reshape(-1, 2)[:, 0].sum())
+        got.append(bos.to_host(b.out, recs.dtype))
+    assert (digest[0] != digest[1]) == streams
+    np.testing.assert_array_equal(got[0], got[1])
+    for j in (0, count - 1):
+        ref, _ = oracle.orp(recs[j * n:(j + 1) * n], Z, int(seeds[j]), method=oracle.CLOSED)
+        np.testing.assert_array_equal(got[0][j * n:(j + 1) * n], ref)
