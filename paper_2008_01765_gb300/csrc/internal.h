@@ -111,7 +111,6 @@ cudaError_t launch_perm_table_batched(const BatchLast* args, const uint2* units,
 
 // Streaming first / middle ORP pass (orp_stream.cu): one CTA per subproblem, input buckets
 // through a TMA ring, output chunks write-combined in shared memory; Z a multiple of 32, <= 2048.
-uint32_t orp_stream_smem_bytes(int R, uint32_t Z, uint32_t k, bool first);
 // Most levels a streaming pass holds in smem_limit bytes (0: the kernel cannot take this Z).
 uint32_t orp_stream_max_k(int R, uint32_t Z, bool first, uint32_t smem_limit);
 inline uint32_t orp_stream_min_k() { return 5; }  // of a caller-given k; automatic plans go down to 4
@@ -174,7 +173,7 @@ uint64_t radix_tiles(uint64_t n, int R);
 
 // Hybrid radix sort (sort_hybrid.cu): MSD partitions on the top one or two digits, then an on-chip
 // sort of every range of groups; falls back to the LSD passes (ctrl->sort_mode = 0) when a group
-// exceeds hybrid_cap(R) records. stage: 0 histogram (hist and joint), 1 plan, 2 partition by the
+// exceeds Local<R>::kCap records. stage: 0 histogram (hist and joint), 1 plan, 2 partition by the
 // top varying digit, 3 partition by the next one inside every bucket, 4 the on-chip sort.
 constexpr uint32_t kSortClasses = 6;
 // What the plan kernel tells the host (mapped pinned memory): the host launches only the passes and the
@@ -203,7 +202,6 @@ struct HybridArgs {
   uint32_t host_seq;
   Ctrl* ctrl;
 };
-uint32_t hybrid_cap(int R);
 uint32_t hybrid_local_ctas(uint64_t n, int R);
 size_t hybrid_spill_bytes(uint64_t n, int R);
 // list (stage 4): ranges of every class (their launches are left out where there are none).

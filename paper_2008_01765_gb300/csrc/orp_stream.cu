@@ -588,11 +588,6 @@ cudaError_t stream_launch(const PassArgs& a, cudaStream_t st) {
 
 }  // namespace
 
-
-uint32_t orp_stream_smem_bytes(int R, uint32_t Z, uint32_t k, bool first) {
-  return stream_layout(R, Z, k, first).total;
-}
-
 uint32_t orp_stream_max_k(int R, uint32_t Z, bool first, uint32_t smem_limit) {
   if (Z % 32 != 0 || Z > kMaxZ) return 0;
   uint32_t best = 0;

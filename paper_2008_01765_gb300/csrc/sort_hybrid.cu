@@ -1526,8 +1526,6 @@ size_t hybrid_spill_bytes(uint64_t n, int R) {
 
 uint32_t batch_sort_cap(int R) { return R == 8 ? Bin<8, kClasses - 2>::kMax : Bin<16, kClasses - 2>::kMax; }
 
-uint32_t hybrid_cap(int R) { return R == 8 ? Local<8>::kCap : Local<16>::kCap; }
-
 cudaError_t launch_hybrid(const HybridArgs& a, int R, int stage, const uint32_t* list, cudaStream_t st) {
   if (a.n == 0) return cudaSuccess;
   return R == 8 ? launch_r<8>(a, stage, list, st) : launch_r<16>(a, stage, list, st);
