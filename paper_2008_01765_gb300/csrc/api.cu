@@ -21,7 +21,7 @@ constexpr uint32_t kMaxPasses = 32;
 constexpr uint32_t kMaxLevels = 32;  // L < 32: slot indexes are 32-bit
 constexpr uint32_t kDefaultAttempts = 8;
 constexpr uint32_t kMaxStreamK = 8;     // most levels of a streaming pass
-constexpr uint32_t kPlanSms = 152;     // SMs the planner counts on
+constexpr uint32_t kPlanSms = 152;     // SMs the planner counts on: GB300's (plans must not need a device)
 constexpr uint32_t kTicketLoads = 20;  // ctrl ticket of the final loads' prefix (0: LAST pass, 1..14: the sort)
 
 // Process-wide debug state. The trace buffer is read once per call under g_state_mu, so an
@@ -545,9 +545,13 @@ bos_status make_plan(uint64_t n, const bos_params* p, bool sort, Plan* pl, uint3
             }
         }
       }
-      // A small array may be quicker on the cluster passes, which spread one subproblem over C SMs.
-      // Measured, ORP of 2^20 16-byte records: Z = 512 170 us against 217, Z = 1024 184 against 307 (the
-      // estimate: 2 ns per slot of a CTA's share; the loads' prefix costs the tile pass about 8 us).
+      // A small array may be quicker on the cluster passes, which spread one subproblem over C SMs (the
+      // estimate: 2 ns per slot of a CTA's share; the loads' prefix costs the tile pass about 8 us). ORP of
+      // 16-byte records, us, streaming split against cluster plan, * taken: Z = 512 2^16 *79 89,
+      // 2^18 120 *98, 2^20 197 *164, 2^21 *258 280, 2^23 *705 861; Z = 1024 2^15 *99 82, 2^18 146 *109,
+      // 2^20 283 *175, 2^22 *403 461. Below Z = 512 the estimate was never fitted and the streaming split
+      // is taken: as good from 2^21 on (Z = 256 2^22 *487 507) and up to 2^16 (81 79), slower in between (2^20
+      // *218 163; Z = 64 2^18 *175 106, and again from 2^22 on: *3809 2918).
       uint32_t snp_max = !bn ? bnp : (double)B * p->Z >= 5e8 ? bn : 0u;  // see below
       if (bn && !p->k && p->Z >= 512 && n < (1u << 22)) {
         double us = 0;
@@ -560,7 +564,10 @@ bos_status make_plan(uint64_t n, const bos_params* p, bool sort, Plan* pl, uint3
       }
       pl->last_tile = bn > 0;
       // streaming passes before the cluster kernel's last one: where the tile's last pass does not do, and
-      // where it saves one of several long passes (2^30 16-byte records at Z = 1024)
+      // where it saves one of several long passes (2^30 16-byte records at Z = 1024 71 ms against 82 with the
+      // tile and a pass more, 2^29 at Z = 256 50 against 67). Between 2^25 and 2^28 records it saves none; on
+      // smaller arrays it pays at Z = 256 (2^22 413 us against 493) and costs elsewhere (Z = 512 440 against
+      // 414, Z = 1024 594 against 409; 2^24 1306 against 1198).
       uint32_t snp = bn;
       for (uint32_t np = 1; ksf && np < snp_max && (np == 1 || ksm); ++np)
         for (uint32_t l = 1; l < L; ++l)
