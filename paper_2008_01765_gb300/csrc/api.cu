@@ -135,8 +135,8 @@ struct Zeroer {
 
 // Host words of the calls in flight: the sort's plan and the control block's copy, in pinned mapped
 // memory (a copy to pageable memory takes 5 us longer, and the plan can be read while the ORP runs).
-// kHostSlots slots, allocated once (4 KiB) by a call that may allocate; a call that finds none free, or no
-// block where it may not allocate one, works without.
+// kHostSlots slots in one block (4 KiB), made by the first call that may allocate and anew after a device
+// reset; a call that finds none free, or no block where it may not make one, works without.
 struct HostSlot {
   HostPlan plan;
   uint32_t pad[7];
